@@ -664,9 +664,13 @@ int run_backward(const bysdf_materials* m, const bysdf_hits* h, int64_t n, const
   }
   a.partials = deterministic ? reinterpret_cast<float*>((uint8_t*)ws + ws_partials_off(m->n_mat))
                              : nullptr;
-  const size_t smem = a.mode == MODE_ALL_SMEM
-                          ? (size_t)m->n_mat * a.sstride + sizeof(float) * np * m->n_mat
-                          : (size_t)(c.block / 32) * m->stride;
+  // tables, and for records in any order the CTA's sums and each warp's list
+  // of its tile's records by material; or one table slot per warp
+  size_t smem = (size_t)(c.block / 32) * m->stride;
+  if (a.mode == MODE_ALL_SMEM) {
+    a.order_off = (int32_t)align_up((size_t)m->n_mat * a.sstride + sizeof(float) * np * m->n_mat, 16);
+    smem = (size_t)a.order_off + kBwdOrderBytes * (size_t)(c.block / 32);
+  }
   if (smem > m->smem_optin) return fail(BYSDF_E_UNSUPPORTED, "material table too large for shared memory");
   if (smem > 48 * 1024) BY_CU(set_backward_smem_limit(c.block, c.occupancy, kind, smem));
   int occ = 0;

@@ -1,19 +1,99 @@
 // Backward kernels of libbysdf.
 //
-// k_backward: per-material parameter gradients.  Recomputes the forward pass
-// of each record with the helix angles as dual-number tangents (the other
-// parameters in closed form) and reduces sum_c g_c df_c/dtheta per material --
-// warp shuffles over a single-material warp tile, then one atomic (or one
-// fixed-order partial) per tile; with unsorted records, shared-memory
-// accumulators per CTA.  KIND: the 8-column basic set, the 15-column
-// extended set, or the basic set with the upstream gradient of an L2 loss
-// (its value a ninth accumulated column, flushed to the per-material loss).
+// k_backward: per-material parameter gradients.  Each record's forward pass
+// is recomputed and differentiated (bysdf_grad.cuh).  KIND: the 8-column basic
+// set, the 15-column extended set, or the basic set with the upstream gradient
+// of an L2 loss (its value a ninth accumulated column, flushed to the
+// per-material loss).
 //
-// k_dirgrad: per-record vector-Jacobian products with respect to the record's
-// directions, forward mode with 6 tangents (wi, wo); no reduction.
+// k_dirgrad: the per-record vector-Jacobian products with respect to the
+// record's directions; no reduction.
+//
+// Reduction.  A warp keeps one material's sums in registers, a partial sum
+// per lane, and flushes them when the material changes: 16 columns are folded
+// across the lanes with 16 shuffles (each step halves the columns a lane
+// holds), then one atomic per column.  Material-sorted tiles change material
+// rarely.  Records in any order are taken by material within the tile (a
+// counting sort across the warp), so that a tile of 512 records of 8
+// materials is flushed 8 times; per-record atomics on shared accumulators,
+// whose lanes meet in a few addresses, cost more than the gradients.
 #include "bysdf_launch.h"
 
 namespace bysdf {
+
+// Sums of each of NP (<= 16) per-lane columns over the warp; lane k returns
+// column k's sum (0 for k >= NP).  Step o hands the half of the columns that
+// the partner keeps to it, so the steps cost 8, 4, 2, 1 shuffles, and one more
+// adds the two lanes that hold the same column.
+template <int NP>
+__device__ __forceinline__ float warp_columns(const float* acc, int lane) {
+  float v[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) v[k] = k < NP ? acc[k] : 0.f;
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) {
+    const bool hi = (lane & o) != 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      if (k < o) {
+        const float give = hi ? v[k] : v[k + o], keep = hi ? v[k + o] : v[k];
+        v[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+      }
+    }
+  }
+  const float s = v[0] + __shfl_xor_sync(0xffffffffu, v[0], 16);
+  return lane < 16 ? s : 0.f;
+}
+
+// Records of a tile in any material order, listed by material (`shift` drops
+// low bits of the id when there are more than 32: records of one bucket then
+// come in any order, which the flush allows).  Ids out of range are listed
+// with material 0 (they contribute nothing).
+__device__ __forceinline__ void material_order(const KArgs& a, int64_t begin, int64_t end,
+                                               int lane, uint16_t* list, uint32_t* hist) {
+  const int count = (int)(end - begin);
+  const uint32_t lt = (1u << lane) - 1u;
+  int shift = 0;
+  while (((a.n_mat - 1) >> shift) >= 32) ++shift;
+  auto bucket = [&](int e) {
+    int mm = __ldg(a.mat_id + begin + e);
+    mm = (mm >= 0 && mm < a.n_mat) ? mm : 0;
+    return (uint32_t)(mm >> shift);
+  };
+  hist[lane] = 0u;
+  __syncwarp();
+#pragma unroll 1
+  for (int e0 = 0; e0 < count; e0 += 32) {
+    const int e = e0 + lane;
+    const uint32_t b = e < count ? bucket(e) : 32u;
+    const uint32_t peers = __match_any_sync(0xffffffffu, b);
+    if (b < 32u && lane == __ffs(peers) - 1) hist[b] += (uint32_t)__popc(peers);
+    __syncwarp();
+  }
+  // exclusive scan of the bucket counts (lane = bucket)
+  const uint32_t h = hist[lane];
+  uint32_t incl = h;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  hist[lane] = incl - h;
+  __syncwarp();
+#pragma unroll 1
+  for (int e0 = 0; e0 < count; e0 += 32) {
+    const int e = e0 + lane;
+    const uint32_t b = e < count ? bucket(e) : 32u;
+    const uint32_t peers = __match_any_sync(0xffffffffu, b);
+    const uint32_t base = b < 32u ? hist[b] : 0u;
+    __syncwarp();
+    if (b < 32u) {
+      list[base + (uint32_t)__popc(peers & lt)] = (uint16_t)e;
+      if (lane == __ffs(peers) - 1) hist[b] = base + (uint32_t)__popc(peers);
+    }
+    __syncwarp();
+  }
+}
 
 template <int BLOCK, int MINB, int KIND>
 __global__ void __launch_bounds__(BLOCK, MINB) k_backward(const KArgs a) {
@@ -21,71 +101,100 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_backward(const KArgs a) {
   constexpr int NG = KbCols<KIND>::grad;     // gradient columns of grad_params
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ uint64_t bars[2 * (BLOCK / 32)];
-  // MODE_ALL_SMEM: per-CTA accumulators behind the tables
+  // records in any order: per-CTA accumulators behind the tables, then each
+  // warp's record list and bucket counts
   float* sacc = reinterpret_cast<float*>(smem + (size_t)a.n_mat * a.sstride);
-  if (a.mode == MODE_ALL_SMEM) {
+  const bool any_order = a.mode == MODE_ALL_SMEM;
+  if (any_order) {
     for (int k = threadIdx.x; k < a.n_mat * NP; k += BLOCK) sacc[k] = 0.f;
   }
+  uint8_t* mine = smem + a.order_off + (threadIdx.x >> 5) * kBwdOrderBytes;
+  uint32_t* hist = reinterpret_cast<uint32_t*>(mine);
+  uint16_t* list = reinterpret_cast<uint16_t*>(mine + 32 * sizeof(uint32_t));
+  const bool listed = any_order && a.mat_id != nullptr && a.n_mat > 1;
+  float acc[NP];
+#pragma unroll
+  for (int k = 0; k < NP; ++k) acc[k] = 0.f;
+  int cur = -1;  // the material the sums belong to (-1: none yet)
+  auto flush = [&](int lane) {
+    if (cur < 0) return;
+    const float v = warp_columns<NP>(acc, lane);
+#pragma unroll
+    for (int k = 0; k < NP; ++k) acc[k] = 0.f;
+    if (lane >= NP || v == 0.f) return;
+    if (any_order) {
+      atomicAdd(&sacc[cur * NP + lane], v);
+    } else if (lane < NG) {
+      atomicAdd(a.grad_params + (size_t)cur * NG + lane, v);
+    } else if (a.loss_mat) {
+      atomicAdd(a.loss_mat + cur, v);
+    }
+  };
   persistent_loop<BLOCK>(a, smem, bars,
                              [&](int64_t begin, int64_t end, int mat, uint8_t* slot, int lane,
                                  int tile) {
-    float acc[NP];
-#pragma unroll
-    for (int k = 0; k < NP; ++k) acc[k] = 0.f;
+    if (listed) material_order(a, begin, end, lane, list, hist);
+    if (mat >= 0 && cur != mat) {
+      if (!a.partials) flush(lane);
+      cur = mat;
+    }
+    const int count = (int)(end - begin);
     // rolled: one copy of the (large) record body
 #pragma unroll 1
-    for (int64_t i = begin + lane; i < end; i += 32) {
-      if (!bounds_ok(i >= 0 && i < a.n)) continue;
-      Record q;
-      load_record(a, i, true, false, q);
-      // one call site of the (large, dual-number) record body for both
-      // scheduling modes keeps the kernel's code small
-      int mm;
-      const uint8_t* tb;
-      if (mat >= 0) {
-        q.mat = mat;
-        mm = mat;
-        tb = slot;
-      } else {
-        q.mat = a.mat_id ? __ldcg(a.mat_id + i) : 0;
-        mm = (q.mat >= 0 && q.mat < a.n_mat) ? q.mat : 0;
-        tb = smem + (size_t)mm * a.sstride;
-      }
-      const MatDev* m = reinterpret_cast<const MatDev*>(tb);
+    for (int e0 = 0; e0 < count; e0 += 32) {
+      const int e = e0 + lane;
+      bool active = e < count;
+      const int64_t i = begin + (active ? (listed ? (int)list[e] : e) : 0);
+      active = active && bounds_ok(i >= 0 && i < a.n);
+      int mm = 0;
       float g[NP];
-      backward_record<KIND>(a, *m, reinterpret_cast<const float2*>(m + 1), i, q, g);
+#pragma unroll
+      for (int k = 0; k < NP; ++k) g[k] = 0.f;
+      if (active) {
+        Record q;
+        load_record(a, i, true, false, q);
+        const uint8_t* tb;
+        if (mat >= 0) {
+          q.mat = mm = mat;
+          tb = slot;
+        } else {
+          q.mat = a.mat_id ? __ldcg(a.mat_id + i) : 0;
+          mm = (q.mat >= 0 && q.mat < a.n_mat) ? q.mat : 0;
+          tb = smem + (size_t)mm * a.sstride;
+        }
+        const MatDev* m = reinterpret_cast<const MatDev*>(tb);
+        backward_record<KIND, NP>(a, *m, reinterpret_cast<const float2*>(m + 1), i, q, g);
+      }
       if (mat >= 0) {
 #pragma unroll
         for (int k = 0; k < NP; ++k) acc[k] += g[k];
-      } else if (q.mat == mm) {
+        continue;
+      }
+      // the lanes whose record is of the current material add to its sums;
+      // while others are left, the sums are flushed and the next is current
+      bool left = active;
+      for (;;) {
+        const bool add = left && mm == cur;
 #pragma unroll
-        for (int k = 0; k < NP; ++k)
-          if (g[k] != 0.f) atomicAdd(&sacc[mm * NP + k], g[k]);
+        for (int k = 0; k < NP; ++k) acc[k] += add ? g[k] : 0.f;
+        left = left && !add;
+        const unsigned rest = __ballot_sync(0xffffffffu, left);
+        if (!rest) break;
+        flush(lane);
+        cur = __shfl_sync(0xffffffffu, mm, __ffs(rest) - 1);
       }
     }
-    if (mat >= 0) {
+    if (a.partials) {
+      // deterministic: this tile's sums, in a fixed order
+      const float v = warp_columns<NP>(acc, lane);
+      if (lane < NP) a.partials[(size_t)tile * NP + lane] = v;
 #pragma unroll
-      for (int k = 0; k < NP; ++k) {
-        float v = acc[k];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        acc[k] = v;
-      }
-      if (lane == 0) {
-        if (a.partials) {
-#pragma unroll
-          for (int k = 0; k < NP; ++k) a.partials[(size_t)tile * NP + k] = acc[k];
-        } else {
-#pragma unroll
-          for (int k = 0; k < NP; ++k) {
-            if (k < NG) atomicAdd(a.grad_params + (size_t)mat * NG + k, acc[k]);
-            else if (a.loss_mat) atomicAdd(a.loss_mat + mat, acc[k]);
-          }
-        }
-      }
+      for (int k = 0; k < NP; ++k) acc[k] = 0.f;
     }
+    __syncwarp();  // the list is rewritten by the next tile
   });
-  if (a.mode == MODE_ALL_SMEM) {
+  if (!a.partials) flush(threadIdx.x & 31);
+  if (any_order) {
     __syncthreads();
     for (int k = threadIdx.x; k < a.n_mat * NP; k += BLOCK) {
       if (sacc[k] == 0.f) continue;
@@ -123,90 +232,6 @@ __global__ void k_reduce_partials(const KArgs a) {
   }
 }
 
-enum { DD_WI = 0, DD_WO = 3, NDD = 6 };
-
-// A shading state with omega_i's three tangents as one with all six (the
-// omega_o tangents zero).
-template <class D, class DI>
-__device__ __forceinline__ D widen_di(const DI& x) {
-  D r(x.v);
-#pragma unroll
-  for (int k = 0; k < 3; ++k) r.d[DD_WI + k] = x.d[k];
-  return r;
-}
-template <class D, class DI>
-__device__ __forceinline__ V3<D> widen_di3(const V3<DI>& x) {
-  return mk3<D>(widen_di<D>(x.x), widen_di<D>(x.y), widen_di<D>(x.z));
-}
-template <class D, class DI>
-__device__ __forceinline__ Shade<D> widen_shade(const Shade<DI>& x) {
-  Shade<D> r;
-  r.t = widen_di3<D>(x.t);
-  r.b = widen_di3<D>(x.b);
-  r.n = widen_di3<D>(x.n);
-  r.wi = widen_di3<D>(x.wi);
-  r.mui = widen_di<D>(x.mui);
-  r.g = widen_di<D>(x.g);
-  r.fr = widen_di<D>(x.fr);
-  r.at = x.at;
-  r.ab = x.ab;
-  r.at_free = x.at_free;
-  r.ab_free = x.ab_free;
-  r.body_x0 = widen_di<D>(x.body_x0);
-  r.body_y0 = widen_di<D>(x.body_y0);
-  r.ni_sy = x.ni_sy;
-  r.tt_ok = x.tt_ok;
-  r.iy = widen_di3<D>(x.iy);
-  r.by = widen_di3<D>(x.by);
-  r.ny = widen_di3<D>(x.ny);
-  r.tx = widen_di<D>(x.tx);
-  r.tau = widen_di<D>(x.tau);
-  return r;
-}
-
-// Direction vector-Jacobian products of one record: sum_c g_c df_c/dwi and
-// df_c/dwo.  Tangents 0..2: wi, 3..5: wo.  The material's helix angles carry
-// no tangent here; the float pre-pass of the geometry picks each node's ply.
-__device__ __forceinline__ void dirgrad_record(const KArgs& a, const MatDev& m,
-                                               const float2* map, int64_t i, Record& q,
-                                               float gwi[3], float gwo[3]) {
-  typedef DualF<NDD> D;
-  typedef DualF<3> DI;   // omega_i's tangents alone
-#pragma unroll
-  for (int c = 0; c < 3; ++c) gwi[c] = gwo[c] = 0.f;
-  if (!record_valid(q, a.n_mat, true, a.ratio != nullptr, false)) return;
-  // omega_o enters only the lobes: the geometry and the shading frame carry
-  // omega_i's three tangents, and are widened to all six for the lobes
-  const MatVars<DI> mv = mat_vars<DI>(m, false);
-  V3<DI> wi = lift3<DI>(q.wi[0], q.wi[1], q.wi[2]);
-  wi.x.d[0] = 1.f;
-  wi.y.d[1] = 1.f;
-  wi.z.d[2] = 1.f;
-  Geo<DI> G;
-  geometry_k<1, DI, DI>(m, map, mv, q, wi, G);
-  if (G.status != ST_OK) return;
-  Shade<DI> si;
-  make_shade(m, mv, G, wi, si);
-  const Shade<D> s = widen_shade<D>(si);
-  V3<D> wo = lift3<D>(q.wo[0], q.wo[1], q.wo[2]);
-  wo.x.d[DD_WO + 0] = 1.f;
-  wo.y.d[DD_WO + 1] = 1.f;
-  wo.z.d[DD_WO + 2] = 1.f;
-  LobeVals<D> L;
-  eval_lobes(m, s, wo, L);
-  const int64_t n = a.n;
-  const float g0 = __ldg(a.grad_f + i), g1 = __ldg(a.grad_f + n + i),
-              g2 = __ldg(a.grad_f + 2 * n + i);
-  const float* kb = L.refl ? m.alb : m.alb_y;
-  const float gs = g0 + g1 + g2;
-  const float gb = g0 * kb[0] + g1 * kb[1] + g2 * kb[2];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    gwi[c] = gs * L.spec.d[DD_WI + c] + gb * L.body.d[DD_WI + c];
-    gwo[c] = gs * L.spec.d[DD_WO + c] + gb * L.body.d[DD_WO + c];
-  }
-}
-
 template <int BLOCK, int MINB>
 __global__ void __launch_bounds__(BLOCK, MINB) k_dirgrad(const KArgs a) {
   extern __shared__ __align__(128) uint8_t smem[];
@@ -229,13 +254,13 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_dirgrad(const KArgs a) {
         tb = smem + (size_t)mm * a.sstride;
       }
       const MatDev* m = reinterpret_cast<const MatDev*>(tb);
-      float gwi[3], gwo[3];
-      dirgrad_record(a, *m, reinterpret_cast<const float2*>(m + 1), i, q, gwi, gwo);
+      float g[6];
+      backward_record<KB_DIRS, 6>(a, *m, reinterpret_cast<const float2*>(m + 1), i, q, g);
       const int64_t n = a.n;
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        if (a.grad_wi) __stcs(a.grad_wi + c * n + i, gwi[c]);
-        if (a.grad_wo) __stcs(a.grad_wo + c * n + i, gwo[c]);
+        if (a.grad_wi) __stcs(a.grad_wi + c * n + i, g[c]);
+        if (a.grad_wo) __stcs(a.grad_wo + c * n + i, g[3 + c]);
       }
     }
   });

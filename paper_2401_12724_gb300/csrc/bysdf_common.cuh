@@ -1,5 +1,5 @@
-// Shared device definitions of libbysdf: the per-material table layout, a
-// forward-mode dual number for the backward kernels, and small vector math.
+// Shared device definitions of libbysdf: the per-material table layout, the
+// kernels' own math functions and small vector math.
 #pragma once
 
 #include <cstdint>
@@ -73,12 +73,6 @@ __host__ __device__ inline const uint8_t* mig_table(const MatDev& m) {
 // key word 1 of the migration map choice
 constexpr uint64_t kMigKey1 = 0xB15DF000F1BE0002ull;
 
-// Parameter slots carried by the dual numbers of the backward kernel: the two
-// helix angles, which move the whole geometry.  Albedo (linear), shadow
-// density (only through G = exp(-sigma_s occlusion)) and roughness (only
-// through GGX D and Smith G1) are differentiated in closed form.
-enum { D_ALPHA_P = 0, D_ALPHA_F = 1, ND = 2 };
-
 // ------------------------------------------------------------- randomness --
 // Philox4x64-10 (Salmon, Moraes, Dror, Shaw, SC 2011): ten rounds of two
 // 64 x 64 -> 128-bit products of the counter words, the key bumped by the
@@ -119,130 +113,15 @@ struct StochCtx {
   uint64_t seed, index;
 };
 
-// ------------------------------------------------------------ dual numbers --
-template <int N>
-struct DualF {
-  float v;
-  float d[N];
-  DualF() = default;
-  __device__ __forceinline__ DualF(float x) : v(x) {
-#pragma unroll
-    for (int k = 0; k < N; ++k) d[k] = 0.f;
-  }
-};
-
-template <class S> struct is_dual { static constexpr bool value = false; };
-template <int N> struct is_dual<DualF<N>> { static constexpr bool value = true; };
-
-__device__ __forceinline__ float vf(float x) { return x; }
-template <int N> __device__ __forceinline__ float vf(const DualF<N>& x) { return x.v; }
-
-#define BY_DF template <int N> __device__ __forceinline__ DualF<N>
-BY_DF operator+(const DualF<N>& a, const DualF<N>& b) {
-  DualF<N> r;
-  r.v = a.v + b.v;
-#pragma unroll
-  for (int k = 0; k < N; ++k) r.d[k] = a.d[k] + b.d[k];
-  return r;
-}
-BY_DF operator-(const DualF<N>& a, const DualF<N>& b) {
-  DualF<N> r;
-  r.v = a.v - b.v;
-#pragma unroll
-  for (int k = 0; k < N; ++k) r.d[k] = a.d[k] - b.d[k];
-  return r;
-}
-BY_DF operator-(const DualF<N>& a) {
-  DualF<N> r;
-  r.v = -a.v;
-#pragma unroll
-  for (int k = 0; k < N; ++k) r.d[k] = -a.d[k];
-  return r;
-}
-BY_DF operator*(const DualF<N>& a, const DualF<N>& b) {
-  DualF<N> r;
-  r.v = a.v * b.v;
-#pragma unroll
-  for (int k = 0; k < N; ++k) r.d[k] = fmaf(a.d[k], b.v, a.v * b.d[k]);
-  return r;
-}
-BY_DF operator/(const DualF<N>& a, const DualF<N>& b) {
-  DualF<N> r;
-  const float inv = 1.0f / b.v;
-  r.v = a.v * inv;
-#pragma unroll
-  for (int k = 0; k < N; ++k) r.d[k] = (a.d[k] - r.v * b.d[k]) * inv;
-  return r;
-}
-BY_DF operator+(const DualF<N>& a, float b) {
-  DualF<N> r = a;
-  r.v += b;
-  return r;
-}
-BY_DF operator+(float a, const DualF<N>& b) { return b + a; }
-BY_DF operator-(const DualF<N>& a, float b) {
-  DualF<N> r = a;
-  r.v -= b;
-  return r;
-}
-BY_DF operator-(float a, const DualF<N>& b) {
-  DualF<N> r;
-  r.v = a - b.v;
-#pragma unroll
-  for (int k = 0; k < N; ++k) r.d[k] = -b.d[k];
-  return r;
-}
-BY_DF operator*(const DualF<N>& a, float b) {
-  DualF<N> r;
-  r.v = a.v * b;
-#pragma unroll
-  for (int k = 0; k < N; ++k) r.d[k] = a.d[k] * b;
-  return r;
-}
-BY_DF operator*(float a, const DualF<N>& b) { return b * a; }
-BY_DF operator/(const DualF<N>& a, float b) { return a * (1.0f / b); }
-BY_DF operator/(float a, const DualF<N>& b) {
-  DualF<N> r;
-  const float inv = 1.0f / b.v;
-  r.v = a * inv;
-  const float g = -r.v * inv;
-#pragma unroll
-  for (int k = 0; k < N; ++k) r.d[k] = g * b.d[k];
-  return r;
-}
-template <int N>
-__device__ __forceinline__ DualF<N> dchain(const DualF<N>& a, float fv, float g) {
-  DualF<N> r;
-  r.v = fv;
-#pragma unroll
-  for (int k = 0; k < N; ++k) r.d[k] = g * a.d[k];
-  return r;
-}
-
-// ------------------------------------------------------- math, float + dual --
+// -------------------------------------------------------------------- math --
 __device__ __forceinline__ float xsqrt(float x) { return sqrtf(x); }
-BY_DF xsqrt(const DualF<N>& a) {
-  const float s = sqrtf(a.v);
-  return dchain(a, s, s > 0.f ? 0.5f / s : 0.f);
-}
-// 1 / sqrt(x).  Floats: the square root and the division (measured 1%
-// faster in the forward kernels than rsqrtf).  Duals: the hardware
-// reciprocal square root and the chain rule (the backward 2.7% faster than
-// with a square root and a division).
+// 1 / sqrt(x) by the square root and the division (measured 1% faster in the
+// forward kernels than rsqrtf).
 __device__ __forceinline__ float xrsqrt(float x) { return 1.0f / sqrtf(x); }
-BY_DF xrsqrt(const DualF<N>& a) {
-  const float r = rsqrtf(a.v);
-  return dchain(a, r, -0.5f * r * r * r);
-}
 // hardware exp2 / log2 based (relative error ~1e-7 for the arguments here,
-// |x| < ~20), for floats and for the values of duals alike
+// |x| < ~20)
 __device__ __forceinline__ float xexp(float x) { return __expf(x); }
-BY_DF xexp(const DualF<N>& a) {
-  const float e = __expf(a.v);
-  return dchain(a, e, e);
-}
 __device__ __forceinline__ float xlog(float x) { return __logf(x); }
-BY_DF xlog(const DualF<N>& a) { return dchain(a, __logf(a.v), 1.0f / a.v); }
 // atan2 for the float path: the octant's ratio a = min(|x|, |y|) / max(|x|,
 // |y|) in [0, 1], atan(a) = a P(a^2) with P of degree 8 (coefficients fitted
 // here by weighted least squares on Chebyshev nodes of [0, 1]; maximum
@@ -268,15 +147,6 @@ __device__ __forceinline__ float xatan2(float y, float x) {
   if (ay > ax) r = 1.5707963705062866f - r;
   if (x < 0.f) r = 3.1415927410125732f - r;
   return y < 0.f ? -r : r;
-}
-template <int N>
-__device__ __forceinline__ DualF<N> xatan2(const DualF<N>& y, const DualF<N>& x) {
-  DualF<N> r;
-  r.v = xatan2(y.v, x.v);
-  const float inv = 1.0f / (x.v * x.v + y.v * y.v);
-#pragma unroll
-  for (int k = 0; k < N; ++k) r.d[k] = (x.v * y.d[k] - y.v * x.d[k]) * inv;
-  return r;
 }
 // Sine and cosine of an angle of at most pi/2 in magnitude (the fiber
 // normal's deviation from the ply normal): the Taylor series of sin to
@@ -304,40 +174,18 @@ __device__ __forceinline__ void xsincos(float x, float* s, float* c) {
   *s = fmaf(x * x2, ps, x);
   *c = fmaf(x2, pc, 1.0f);
 }
-template <int N>
-__device__ __forceinline__ void xsincos(const DualF<N>& x, DualF<N>* s, DualF<N>* c) {
-  float sv, cv;
-  xsincos(x.v, &sv, &cv);
-  *s = dchain(x, sv, cv);
-  *c = dchain(x, cv, -sv);
-}
 // sin and cos of 2 pi t (t in turns); the pi-scaled form reduces exactly.
 __device__ __forceinline__ void xsincos_turns(float t, float* s, float* c) {
   sincospif(2.0f * t, s, c);
 }
-template <int N>
-__device__ __forceinline__ void xsincos_turns(const DualF<N>& t, DualF<N>* s, DualF<N>* c) {
-  float sv, cv;
-  sincospif(2.0f * t.v, &sv, &cv);
-  *s = dchain(t, sv, 2.0f * kPi * cv);
-  *c = dchain(t, cv, -2.0f * kPi * sv);
-}
 // sin and cos of 2 pi t for the small per-step phase advances of the ply
 // trace: t is reduced to [-1/2, 1/2] exactly and the hardware
-// approximations are taken (absolute error ~5e-7); the tangents follow from
-// those values.
+// approximations are taken (absolute error ~5e-7).
 __device__ __forceinline__ void xsincos_turns_fast(float t, float* s, float* c) {
   const float r = t - rintf(t);
   __sincosf((2.0f * kPi) * r, s, c);
 }
-template <int N>
-__device__ __forceinline__ void xsincos_turns_fast(const DualF<N>& t, DualF<N>* s, DualF<N>* c) {
-  float sv, cv;
-  xsincos_turns_fast(t.v, &sv, &cv);
-  *s = dchain(t, sv, 2.0f * kPi * cv);
-  *c = dchain(t, cv, -2.0f * kPi * sv);
-}
-template <class S> __device__ __forceinline__ S xmax0(const S& a) { return vf(a) < 0.f ? S(0.f) : a; }
+__device__ __forceinline__ float xmax0(float a) { return a < 0.f ? 0.f : a; }
 
 // ----------------------------------------------------------- index checks --
 // The index-checking build (-DBYSDF_DEBUG_BOUNDS, a separate library, the
@@ -401,26 +249,8 @@ template <class S> __device__ __forceinline__ V3<S> operator-(const V3<S>& a) {
 template <class S, class T> __device__ __forceinline__ V3<S> operator*(const V3<S>& a, const T& s) {
   return mk3<S>(a.x * s, a.y * s, a.z * s);
 }
-// a float vector may meet a dual one (a direction without tangents against
-// the frame): the products then carry only the dual side's tangents
-template <class A, class B> __device__ __forceinline__ auto dot(const V3<A>& a, const V3<B>& b) {
+template <class S> __device__ __forceinline__ S dot(const V3<S>& a, const V3<S>& b) {
   return a.x * b.x + a.y * b.y + a.z * b.z;
-}
-template <int N>
-__device__ __forceinline__ V3<DualF<N>> operator+(const V3<DualF<N>>& a, const V3<float>& b) {
-  return mk3<DualF<N>>(a.x + b.x, a.y + b.y, a.z + b.z);
-}
-template <int N>
-__device__ __forceinline__ V3<DualF<N>> operator+(const V3<float>& a, const V3<DualF<N>>& b) {
-  return mk3<DualF<N>>(a.x + b.x, a.y + b.y, a.z + b.z);
-}
-// a float vector as S (no tangents), or the vector itself
-template <class S, class W> __device__ __forceinline__ V3<S> as3(const V3<W>& w) {
-  if constexpr (std::is_same<S, W>::value) {
-    return w;
-  } else {
-    return mk3<S>(S(w.x), S(w.y), S(w.z));
-  }
 }
 template <class S> __device__ __forceinline__ V3<S> cross(const V3<S>& a, const V3<S>& b) {
   return mk3<S>(a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x);

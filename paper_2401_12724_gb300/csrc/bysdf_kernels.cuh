@@ -3,7 +3,7 @@
 // loads, the warp-granular tile queue, and the per-record drivers.
 #pragma once
 
-#include "bysdf_model.cuh"
+#include "bysdf_grad.cuh"
 
 namespace bysdf {
 
@@ -62,7 +62,7 @@ struct KArgs {
   const float* weight;   // L2 backward: per-record loss weights, or NULL (1)
   float* loss_mat;       // L2 backward: per-material loss, or NULL
   int32_t n_param;       // gradient columns: 8, or 15 (extended set)
-  int32_t order_off;      // forward: byte offset of the warps' sort keys in shared memory
+  int32_t order_off;      // byte offset of the warps' order lists in shared memory
   float *grad_wi, *grad_wo;  // direction backward: 3 planes each, or NULL
   uint64_t stoch_seed;       // stochastic estimators: generator key word 0,
   int64_t stoch_index0;      //   global index of record 0,
@@ -189,14 +189,14 @@ __device__ __forceinline__ void forward_record(const KArgs& a, const MatDev& m,
   const bool eval_ok = base && (!kEval || unit_ok(q.wo));
   const bool samp_ok = base && (!kSample || u_valid(q));
   int st = ST_INVALID;
-  Geo<float> G;
-  Shade<float> s;
+  Geo G;
+  Shade s;
   if (eval_ok || samp_ok) {
-    const MatVars<float> mv = mat_vars<float>(m);
+    const MatVars mv = mat_vars(m);
     if constexpr ((OP & OPF_STOCH) != 0) {
       const StochCtx sc{a.stoch_flags, a.stoch_seed, (uint64_t)(a.stoch_index0 + i)};
       const V3<float> wi = mk3<float>(q.wi[0], q.wi[1], q.wi[2]);
-      geometry_k<PLIES, float, float>(m, map, mv, q, wi, G, &sc);
+      geometry_k<PLIES>(m, map, mv, q, wi, G, &sc);
       st = G.status;
       if (st == ST_OK) make_shade(m, mv, G, wi, s, &sc);
     } else {
@@ -209,7 +209,7 @@ __device__ __forceinline__ void forward_record(const KArgs& a, const MatDev& m,
     float f0 = 0.f, f1 = 0.f, f2 = 0.f, p = 0.f;
     const int est = eval_ok ? st : ST_INVALID;
     if (est == ST_OK) {
-      LobeVals<float> L;
+      LobeVals L;
       eval_lobes(m, s, mk3<float>(q.wo[0], q.wo[1], q.wo[2]), L);
       const float* kb = L.refl ? m.alb : m.alb_y;  // k^B_x (Eq. 5) or k^B_y (Eq. 6)
       f0 = L.spec + kb[0] * L.body;
@@ -240,7 +240,7 @@ __device__ __forceinline__ void forward_record(const KArgs& a, const MatDev& m,
         w0 = wo.x;
         w1 = wo.y;
         w2 = wo.z;
-        LobeVals<float> L;
+        LobeVals L;
         eval_lobes(m, s, wo, L);
         const float pt = total_pdf(m, s, L);
         if (pt > 0.f) {
@@ -265,99 +265,46 @@ __device__ __forceinline__ void forward_record(const KArgs& a, const MatDev& m,
   }
 }
 
-// Kinds of the backward: the 8 parameters of the basic set, the 15 of the
-// extended set, and the basic set with the upstream gradient taken from an
-// L2 loss against target radiance, whose value is a ninth column.
-enum { KB_BASIC = 0, KB_EXT = 1, KB_L2 = 2 };
-template <int KIND> struct KbCols {
-  static constexpr int grad = KIND == KB_EXT ? 15 : 8;            // gradient columns
-  static constexpr int acc = KIND == KB_L2 ? 9 : grad;             // accumulated columns
-};
-
-// Gradient of sum_c g_c f_c of one record w.r.t. the material parameters:
-// the 8 of the basic set ([0..2] moves both body colours), or the 15 of the
-// extended set (KB_EXT; layout of bysdf_set_params_ext).  KB_L2: g_c =
-// 2 w (f_c - target_c) from the record's own f (Sec. 5.2 fitting of an L2
-// loss), gout[8] = w sum_c (f_c - target_c)^2, and f is written to
-// a.f_rgb when given (0 where the record has no valid evaluation).
-template <int KIND>
+// Gradient of one record (record_grad; N outputs) with its upstream gradient
+// from grad_f, or for KB_L2 g_c = 2 w (f_c - target_c) from the record's own
+// f (Sec. 5.2 fitting of an L2 loss); f is then written to a.f_rgb when given
+// (0 where the record has no valid evaluation).
+template <int KIND, int N>
 __device__ __forceinline__ void backward_record(const KArgs& a, const MatDev& m,
                                                 const float2* map, int64_t i, Record& q,
                                                 float* gout) {
-  typedef DualF<ND> D;
-  constexpr bool EXT = KIND == KB_EXT;
-  constexpr int NA = KbCols<KIND>::acc;
-#pragma unroll
-  for (int k = 0; k < NA; ++k) gout[k] = 0.f;
-  if constexpr (KIND == KB_L2) {
-    if (a.f_rgb) {
-      a.f_rgb[i] = 0.f;
-      a.f_rgb[a.n + i] = 0.f;
-      a.f_rgb[2 * a.n + i] = 0.f;
-    }
-  }
-  if (!record_valid(q, a.n_mat, true, a.ratio != nullptr, false)) return;
-  const MatVars<D> mv = mat_vars<D>(m);
-  Geo<D> G;
-  // one ply per pass in the float pick pass: fewer live registers at the
-  // backward's 128 (2.6% faster than two)
-  geometry<1>(m, map, mv, q, G);
-  if (G.status != ST_OK) return;
-  Shade<D> s;
-  make_shade(m, mv, G, q, s);
-  LobeVals<D> L;
-  float dln_a[2] = {0.f, 0.f};
-  eval_lobes(m, s, mk3<float>(q.wo[0], q.wo[1], q.wo[2]), L, dln_a);
   const int64_t n = a.n;
-  // f_c = spec + k^B_c body, with k^B = k^B_x (reflection side) or k^B_y
-  const float* kb = L.refl ? m.alb : m.alb_y;
-  float g0, g1, g2;
-  if constexpr (KIND == KB_L2) {
-    const float f0 = L.spec.v + kb[0] * L.body.v, f1 = L.spec.v + kb[1] * L.body.v,
-                f2 = L.spec.v + kb[2] * L.body.v;
-    if (a.f_rgb) {
-      a.f_rgb[i] = f0;
-      a.f_rgb[n + i] = f1;
-      a.f_rgb[2 * n + i] = f2;
-    }
-    const float w = a.weight ? __ldcg(a.weight + i) : 1.0f;
-    const float d0 = f0 - __ldcg(a.target + i), d1 = f1 - __ldcg(a.target + n + i),
-                d2 = f2 - __ldcg(a.target + 2 * n + i);
-    g0 = 2.0f * w * d0;
-    g1 = 2.0f * w * d1;
-    g2 = 2.0f * w * d2;
-    gout[8] = w * (d0 * d0 + d1 * d1 + d2 * d2);
-  } else {
-    g0 = __ldcg(a.grad_f + i);
-    g1 = __ldcg(a.grad_f + n + i);
-    g2 = __ldcg(a.grad_f + 2 * n + i);
+#pragma unroll
+  for (int k = 0; k < N; ++k) gout[k] = 0.f;
+  float f[3] = {0.f, 0.f, 0.f};
+  if (record_valid(q, a.n_mat, true, a.ratio != nullptr, false)) {
+    record_grad<KIND>(
+        m, map, q,
+        [&](const float* fc, float* gc) {
+          if constexpr (KIND == KB_L2) {
+            const float w = a.weight ? __ldcg(a.weight + i) : 1.0f;
+            float loss = 0.f;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+              f[c] = fc[c];
+              const float d = fc[c] - __ldcg(a.target + c * n + i);
+              gc[c] = 2.0f * w * d;
+              loss = fmaf(d, d, loss);
+            }
+            return w * loss;
+          } else {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) gc[c] = __ldcg(a.grad_f + c * n + i);
+            return 0.f;
+          }
+        },
+        gout);
   }
-  const float gs = g0 + g1 + g2;
-  const float gb = g0 * kb[0] + g1 * kb[1] + g2 * kb[2];
-  const float body = L.body.v;
-  const int c0 = (EXT && !L.refl) ? 9 : 0;
-  gout[c0 + 0] = g0 * body;
-  gout[c0 + 1] = g1 * body;
-  gout[c0 + 2] = g2 * body;
-  // roughness: d spec / d beta = spec * d ln spec / d alpha (alpha = beta +
-  // footprint term, unless clamped)
-  gout[3] = s.at_free ? gs * L.spec.v * dln_a[0] : 0.f;
-  gout[4] = s.ab_free ? gs * L.spec.v * dln_a[1] : 0.f;
-  // helix angles: the dual tangents
-  gout[5] = gs * L.spec.d[D_ALPHA_P] + gb * L.body.d[D_ALPHA_P];
-  gout[6] = gs * L.spec.d[D_ALPHA_F] + gb * L.body.d[D_ALPHA_F];
-  // shadow density: the body lobes are proportional to G
-  const float Gv = G.g.v;
-  gout[7] = Gv > 0.f ? gb * body * (G.dg_dsig / Gv) : 0.f;
-  if constexpr (EXT) {
-    // body = r B body_w (reflection side) or (1 - r) B body_w; spec = (1 - B)
-    // k_spec spec_u; the transmission lobe carries tau = exp(-sigma_t N_i
-    // |x - y|) (Eq. 4)
-    const float bw = L.body_w.v, su = L.spec_u.v;
-    gout[8] = gb * (L.refl ? m.B : -m.B) * bw;
-    gout[12] = L.refl ? 0.f : gs * L.spec.v * (-s.ni_sy);
-    gout[13] = gb * (L.refl ? m.r : 1.0f - m.r) * bw - gs * m.k_spec * su;
-    gout[14] = gs * (1.0f - m.B) * su;
+  if constexpr (KIND == KB_L2) {
+    if (a.f_rgb) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) __stcs(a.f_rgb + c * n + i, f[c]);
+    }
   }
 }
 
@@ -552,6 +499,11 @@ __device__ __forceinline__ void persistent_loop(const KArgs& a, uint8_t* smem, u
 // lane `lane`; ITEMS items per lane; records past the tile's end are
 // listed as empty).
 constexpr int kOrderBuckets = 32;
+
+// Shared memory per warp of the backward's list of a tile's records by
+// material: 32 bucket counts, then up to 512 places in the tile.
+constexpr int kBwdMaxTile = 512;
+constexpr size_t kBwdOrderBytes = 32 * sizeof(uint32_t) + kBwdMaxTile * sizeof(uint16_t);
 
 // Bucket of a record with a footprint: footprint nodes K (up to 16 told
 // apart), then N_p above or below 4.
