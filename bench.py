@@ -503,7 +503,7 @@ def main():
                                      "'workloads'",
                             step="fused eval(+pdf at wo) + one importance sample per record",
                             l2="inputs larger than L2 (~0.8 GB of records per step)",
-                            launch=M.launch_config(N.OP_FUSED),
+                            launch="640 x 4, the default for records without a footprint",
                             parallelism=f"records sharded, {ws} rank(s)"),
                 # one fused kernel per step: the records come in any order, so no
                 # tile-plan kernel runs (the ncu launch list of this step shows one)

@@ -139,9 +139,10 @@ typedef struct bysdf_hits {
 typedef struct bysdf_launch_config {
   int32_t block;          /* threads per CTA: 128, 256 or 512               */
   int32_t items;          /* records per lane per warp tile: 1, 2, 4 or 8
-                             (the backward also 16); a batch of fewer tiles
-                             than the grid's resident warps takes smaller
-                             tiles, so that more warps get work              */
+                             (the backward also 16); the last tiles of a
+                             batch, and all tiles of one with few tiles per
+                             resident warp, are smaller, so that more warps
+                             get work and end together                       */
   int32_t ctas_per_sm;    /* resident CTAs per SM the grid is sized for
                              (0: as many as fit)                             */
   int32_t occupancy;      /* register budget: 0 the default, 1 a tighter cap
@@ -361,10 +362,12 @@ int bysdf_plain(int op, const bysdf_materials* m, const bysdf_hits* hits,
                 uint8_t* status, void* stream);
 
 /* Launch shape used for op (BYSDF_OP_*), per table.  Until one is set here
- * or by bysdf_autotune, the forward calls take 512 x 4 at occupancy 0 for
- * records without a footprint and 256 x 8 at occupancy 1 for records with a
- * ratio plane (up to 16 geometry nodes each); once set, the shape serves
- * both kinds.  get returns the set shape, else the first default. */
+ * or by bysdf_autotune, the forward calls take 640 x 4 for records without a
+ * footprint (a shape of its own that cannot be set; 512 x 4 at occupancy 0
+ * for the stochastic calls and for sorted records whose tables leave no room
+ * for 20 warps) and 256 x 8 at occupancy 1 for records with a ratio plane (up
+ * to 16 geometry nodes each); once set, the shape serves both kinds.  get
+ * returns the set shape, else 512 x 4 (the backward: 512 x 8). */
 int bysdf_set_launch_config(bysdf_materials* m, int op, const bysdf_launch_config* cfg);
 int bysdf_get_launch_config(const bysdf_materials* m, int op, bysdf_launch_config* cfg);
 
@@ -409,7 +412,7 @@ int bysdf_plain_fused(const bysdf_materials* m, const bysdf_hits* hits,
                       const int64_t* seg_offsets_host, const float* u0, const float* u1,
                       int64_t n, const bysdf_outputs* out, void* stream);
 
-/* Time every supported launch shape of op (BYSDF_OP_EVAL, _SAMPLE, _PDF,
+/* Time every launch shape that can be set for op (BYSDF_OP_EVAL, _SAMPLE, _PDF,
  * _FUSED, _BACKWARD) on these records with CUDA events on `stream`, keep the
  * fastest in the table for later calls and return it in *best.  Writes the
  * op's outputs (several times).  Synchronises the stream; not capturable. */

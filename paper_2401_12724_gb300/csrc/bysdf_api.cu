@@ -28,9 +28,7 @@ struct bysdf_materials {
   std::vector<bysdf_material_desc> desc;
   bysdf_launch_config cfg[BYSDF_NOPS];
   bool cfg_set[BYSDF_NOPS] = {};  // chosen by the caller or by bysdf_autotune
-  // resident CTAs per SM of the forward launch shapes met so far, keyed by
-  // (op bits, block, items, occupancy, dynamic shared memory): the query is
-  // host time that a small batch would otherwise pay on every call
+  // resident CTAs per SM of the launch shapes met so far (cached_shape)
   struct OccEntry {
     int bits, block, items, occ;
     size_t smem;
@@ -356,18 +354,21 @@ size_t ws_tile_start_off() { return kWsCtl; }
 size_t ws_partials_off(int n_mat) { return align_up(kWsCtl + 4 * (size_t)(n_mat + 1), 256); }
 int64_t max_tiles(int64_t n, int n_mat) { return (n + 31) / 32 + n_mat; }
 
-// Defaults measured on GB300 with the benchmark workloads (eval + sample +
-// pdf over 2^24 records; forward + backward over 2^24 material-sorted
-// records of 64 materials): 16 warps per SM in CTAs of 512; four records
-// per lane per warp tile for the forward calls (two or eight within 0.3%),
-// sixteen for the backward (the fused L2 pass per 2^24 records 2.25 ms,
-// against 2.28 ms at eight, 2.53 ms at four and 3.12 ms at two, at the
-// kernels of their times).  bysdf_autotune refines them for a given record
-// set.
+// Defaults measured on GB300 with the benchmark workloads: 16 warps per SM in
+// CTAs of 512 threads (128 registers); tiles of four rounds of 32 records for
+// the forward calls, eight for the backward (the fused L2 pass over 2^24
+// material-sorted records 1574 us, against 1588 us at sixteen, 1634 us at
+// four and 1741 us at one).  Near-field forward calls take near_default_cfg,
+// records with a footprint footprint_default_cfg.  bysdf_autotune refines
+// them for a given record set.
+// rounds of 32 records in the last tiles of a backward batch (its tiles are
+// flushed per material)
+constexpr int kTailBackward = 2;
+
 bysdf_launch_config default_cfg(int op) {
   bysdf_launch_config c;
   c.block = 512;
-  c.items = op == BYSDF_OP_BACKWARD ? 16 : 4;
+  c.items = op == BYSDF_OP_BACKWARD ? 8 : 4;
   c.ctas_per_sm = 0;  // 0: as many as fit
   c.occupancy = 0;
   return c;
@@ -385,11 +386,38 @@ bysdf_launch_config footprint_default_cfg() {
   return c;
 }
 
+// Near-field records: 20 warps per SM in one CTA of 640 threads (96
+// registers; 128 to 200 bytes of spills) instead of 16 at 124 registers: the
+// kernels wait on fixed-latency chains, and a fifth warp per scheduler fills
+// more of them than the spills cost (2^24 fused records 1517 -> 1472 us, 2^21
+// evals of migrating yarns 156 -> 150 us; 22 warps at 88 registers 1605 us).
+constexpr int kNearBlock = 640;
+bysdf_launch_config near_default_cfg() {
+  bysdf_launch_config c;
+  c.block = kNearBlock;
+  c.items = 4;
+  c.ctas_per_sm = 0;
+  c.occupancy = 0;
+  return c;
+}
+
+// Shared memory of a warp's tile order list.
+size_t order_bytes(int items) {
+  return sizeof(uint32_t) * (32 * (size_t)items + kOrderBuckets);
+}
+
 // The shape of a forward call: the caller's (or the tuned) one when set,
-// else the default for the kind of records.
-bysdf_launch_config fwd_cfg(const bysdf_materials* m, int op, const bysdf_hits* h) {
-  if (m->cfg_set[op] || !h || !h->ratio) return m->cfg[op];
-  return footprint_default_cfg();
+// else the default for the kind of records.  Material-sorted records keep a
+// table slot per warp: tables too large for 20 slots (and the kernel's static
+// shared memory, under 1 KB) take the 16-warp shape.
+bysdf_launch_config fwd_cfg(const bysdf_materials* m, int op, const bysdf_hits* h,
+                            bool stochastic = false) {
+  if (m->cfg_set[op] || !h) return m->cfg[op];
+  if (h->ratio) return footprint_default_cfg();
+  const bysdf_launch_config c = near_default_cfg();
+  const bool fits = (size_t)(c.block / 32) * ((size_t)m->stride + order_bytes(c.items)) + 1024 <=
+                    m->smem_optin;
+  return !stochastic && (!h->seg_offsets || fits) ? c : m->cfg[op];
 }
 
 int check_hits(const bysdf_materials* m, const bysdf_hits* h, bool need_wo, int64_t n) {
@@ -422,7 +450,7 @@ int prepare(const bysdf_materials* m, const bysdf_hits* h, int64_t n, void* ws, 
   a->stride = m->stride;
   a->sstride = smem_stride(m);
   a->n = n;
-  a->tile = 32 * items;
+  a->tile = a->tail = 32 * items;
   a->h = h->h;
   a->u = h->u;
   a->v = h->v;
@@ -439,7 +467,7 @@ int prepare(const bysdf_materials* m, const bysdf_hits* h, int64_t n, void* ws, 
     return fail(BYSDF_E_UNSUPPORTED,
                 "tables do not fit in shared memory: pass material-sorted records with seg_offsets");
   }
-  a->n_tiles = (n + a->tile - 1) / a->tile;
+  a->n_main = a->n_tiles = (n + a->tile - 1) / a->tile;
   if (!ws) return fail(BYSDF_E_WORKSPACE, "workspace is NULL");
   if (!aligned16(ws)) return fail(BYSDF_E_ARG, "workspace not 16-byte aligned");
   if (ws_bytes < ws_need)
@@ -480,16 +508,51 @@ int plan(const bysdf_materials* m, KArgs& a, void* ws, cudaStream_t st, int64_t 
   return BYSDF_OK;
 }
 
-cudaError_t cached_forward_occupancy(const bysdf_materials* m, int bits, int block, int items,
-                                     int occ, size_t smem, int* ctas) {
+// Tiles of a batch in any order over `warps` resident warps: tiles of
+// 32 * items records, but the last items rounds of 32 records per warp in
+// tiles of tail_items rounds, so that the warps end together.  A batch of one
+// sample of 10^6 records is 12.8 rounds a warp: in tiles of 4 the last warps
+// work on a fourth tile while the others wait (90 us; 81 us with the short
+// tiles, which alone cost 4% on large batches: each draw is a round trip to
+// the counter).
+void split_tiles(KArgs& a, int items, int tail_items, int64_t warps) {
+  const int64_t rounds = (a.n + 31) / 32;
+  const int64_t main_rounds = std::max<int64_t>(0, rounds - warps * items);
+  a.tile = 32 * items;
+  a.tail = 32 * tail_items;
+  a.n_main = main_rounds / items;
+  const int64_t rest = a.n - a.n_main * a.tile;
+  a.n_tiles = a.n_main + (rest + a.tail - 1) / a.tail;
+}
+
+// Resident CTAs per SM of a launch shape, with its kernel's shared-memory
+// limit raised (to the device's maximum, whatever the shape: a smaller table
+// must not lower it for a larger one).  Both are host time that every call
+// would pay, so they are looked up once per table and shape.  code: the op
+// bits, or kShapeBackward + kind, or kShapeDirgrad.
+constexpr int kShapeBackward = 0x100, kShapeDirgrad = 0x200;
+cudaError_t cached_shape(const bysdf_materials* m, int code, int block, int items, int occ,
+                         size_t smem, int* ctas) {
   std::lock_guard<std::mutex> lock(m->occ_mu);
   for (const auto& e : m->occ_cache)
-    if (e.bits == bits && e.block == block && e.items == items && e.occ == occ && e.smem == smem) {
+    if (e.bits == code && e.block == block && e.items == items && e.occ == occ && e.smem == smem) {
       *ctas = e.ctas;
       return cudaSuccess;
     }
-  const cudaError_t err = forward_occupancy(bits, block, items, occ, smem, ctas);
-  if (err == cudaSuccess) m->occ_cache.push_back({bits, block, items, occ, smem, *ctas});
+  const bool raise = smem > 48 * 1024;
+  cudaError_t err = cudaSuccess;
+  if (code == kShapeDirgrad) {
+    if (raise) err = set_dirgrad_smem_limit(block, m->smem_optin);
+    if (err == cudaSuccess) err = dirgrad_occupancy(block, smem, ctas);
+  } else if (code & kShapeBackward) {
+    const int kind = code - kShapeBackward;
+    if (raise) err = set_backward_smem_limit(block, occ, kind, m->smem_optin);
+    if (err == cudaSuccess) err = backward_occupancy(block, occ, kind, smem, ctas);
+  } else {
+    if (raise) err = set_forward_smem_limit(code, block, items, occ, m->smem_optin);
+    if (err == cudaSuccess) err = forward_occupancy(code, block, items, occ, smem, ctas);
+  }
+  if (err == cudaSuccess) m->occ_cache.push_back({code, block, items, occ, smem, *ctas});
   return err;
 }
 
@@ -565,28 +628,47 @@ int run_forward(const bysdf_materials* m, int op, const bysdf_hits* h, const flo
   const size_t tables = a.mode == MODE_ALL_SMEM ? (size_t)m->n_mat * a.sstride
                                                 : (size_t)(c.block / 32) * m->stride;
   a.order_off = (int32_t)align_up(tables, 16);
-  auto key_bytes = [&](int items) {
-    return sizeof(uint32_t) * (size_t)(c.block / 32) * (32 * (size_t)items + kOrderBuckets);
-  };
-  size_t smem = (size_t)a.order_off + key_bytes(c.items);
-  if (smem > m->smem_optin) return fail(BYSDF_E_UNSUPPORTED, "material table too large for shared memory");
-  if (smem > 48 * 1024) BY_CU(set_forward_smem_limit(bits, c.block, c.items, c.occupancy, smem));
+  size_t smem = 0;
   int occ = 0;
-  BY_CU(cached_forward_occupancy(m, bits, c.block, c.items, c.occupancy, smem, &occ));
-  // fewer warp tiles than resident warps leaves warps idle: tiles of 32
-  // records spread a small batch over twice (or four times) as many warps
+  auto shape = [&](int items) {
+    smem = (size_t)a.order_off + (size_t)(c.block / 32) * order_bytes(items);
+    return cached_shape(m, bits, c.block, items, c.occupancy, smem, &occ);
+  };
+  if ((size_t)a.order_off + (size_t)(c.block / 32) * order_bytes(c.items) > m->smem_optin)
+    return fail(BYSDF_E_UNSUPPORTED, "material table too large for shared memory");
+  BY_CU(shape(c.items));
   const int64_t warps = (int64_t)grid_for(m, c, occ) * (c.block / 32);
-  if (c.items > 1 && a.n_tiles < warps) {
-    c.items = 1;
-    a.tile = 32;
-    a.n_tiles = (n + 31) / 32;
-    smem = (size_t)a.order_off + key_bytes(1);
-    if (smem > 48 * 1024) BY_CU(set_forward_smem_limit(bits, c.block, 1, c.occupancy, smem));
-    BY_CU(cached_forward_occupancy(m, bits, c.block, 1, c.occupancy, smem, &occ));
+  if (a.mode != MODE_SORTED && !h->ratio && !(bits & OPF_STOCH)) {
+    split_tiles(a, c.items, 1, warps);
+  } else {
+    // footprint tiles stay whole (their order list needs records to choose
+    // from) but get smaller where a batch has few rounds of 32 per warp
+    // (measured from 2 10^4 to 6 10^6 records: at 9 rounds a warp, tiles of 4
+    // take 432 us, of 8 486 us, of 2 490 us; at 36 of 8 1407 us, of 4 1446 us)
+    const int64_t rounds = (n + 31) / 32;
+    int items = c.items, tile = c.items;
+    if (h->ratio && !m->cfg_set[op]) {
+      tile = rounds < 3 * warps ? 1 : rounds < 6 * warps ? 2 : rounds < 12 * warps ? 4 : items;
+      items = tile;
+      // the stochastic kernels keep the tile of one round or of c.items they
+      // are built for (theirs differ in the last bits) and work on less of it
+      if (bits & OPF_STOCH) {
+        items = a.n_tiles < warps ? 1 : c.items;
+        tile = std::min(tile, items);
+      }
+    } else if (a.n_tiles < warps) {
+      items = tile = 1;
+    }
+    if (items != c.items) {
+      c.items = items;
+      BY_CU(shape(c.items));
+    }
+    a.tile = a.tail = 32 * tile;
+    a.n_main = a.n_tiles = (n + a.tile - 1) / a.tile;
   }
   const int grid = grid_for(m, c, occ);
   if ((rc = plan(m, a, ws, st, (int64_t)grid * (c.block / 32)))) return rc;
-  BY_CU(launch_forward(bits, a, c.block, c.occupancy, grid, smem, st));
+  BY_CU(launch_forward(bits, a, c.block, c.items, c.occupancy, grid, smem, st));
   return BYSDF_OK;
 }
 
@@ -672,18 +754,26 @@ int run_backward(const bysdf_materials* m, const bysdf_hits* h, int64_t n, const
     smem = (size_t)a.order_off + kBwdOrderBytes * (size_t)(c.block / 32);
   }
   if (smem > m->smem_optin) return fail(BYSDF_E_UNSUPPORTED, "material table too large for shared memory");
-  if (smem > 48 * 1024) BY_CU(set_backward_smem_limit(c.block, c.occupancy, kind, smem));
   int occ = 0;
-  BY_CU(backward_occupancy(c.block, c.occupancy, kind, smem, &occ));
+  BY_CU(cached_shape(m, kShapeBackward + kind, c.block, 0, c.occupancy, smem, &occ));
   if (!deterministic) BY_CU(cudaMemsetAsync(grad_params, 0, sizeof(float) * ng * m->n_mat, st));
   const int grid = grid_for(m, c, occ);
-  // fewer warp tiles than resident warps leaves warps idle: the tile is
-  // halved until the batch covers them (n / tile tiles for records in any
-  // order; material-sorted records have at least as many)
   const int64_t warps = (int64_t)grid * (c.block / 32);
-  while (c.items > 1 && (n + 32 * c.items - 1) / (32 * c.items) < warps) c.items /= 2;
-  a.tile = 32 * c.items;
-  a.n_tiles = (n + a.tile - 1) / a.tile;
+  const int64_t rounds = (n + 31) / 32;
+  if (a.mode == MODE_SORTED) {
+    // fewer warp tiles than resident warps leaves warps idle: the tile is
+    // halved until the batch covers them (at least rounds / items tiles)
+    while (c.items > 1 && (rounds + c.items - 1) / c.items < warps) c.items /= 2;
+    a.tile = a.tail = 32 * c.items;
+    a.n_main = a.n_tiles = (n + a.tile - 1) / a.tile;
+  } else if (rounds <= warps * c.items) {
+    // one tile per warp, as long as it takes: each tile costs a pass over its
+    // ids and a flush per material (200003 records of 8 materials)
+    c.items = (int)((rounds + warps - 1) / warps);
+    split_tiles(a, c.items, c.items, warps);
+  } else {
+    split_tiles(a, c.items, std::min(c.items, kTailBackward), warps);
+  }
   if ((rc = plan(m, a, ws, st, warps))) return rc;
   BY_CU(launch_backward(a, c.block, c.occupancy, kind, grid, smem, st));
   if (deterministic) BY_CU(launch_reduce_partials(a, st));
@@ -693,10 +783,11 @@ int run_backward(const bysdf_materials* m, const bysdf_hits* h, int64_t n, const
     a.grad_wo = grad_wo;
     const size_t smem_d = a.mode == MODE_ALL_SMEM ? (size_t)m->n_mat * a.sstride
                                                   : (size_t)(c.block / 32) * m->stride;
-    if (smem_d > 48 * 1024) BY_CU(set_dirgrad_smem_limit(c.block, smem_d));
     int occ_d = 0;
-    BY_CU(dirgrad_occupancy(c.block, smem_d, &occ_d));
+    BY_CU(cached_shape(m, kShapeDirgrad, c.block, 0, 0, smem_d, &occ_d));
     const int grid_d = grid_for(m, c, occ_d);
+    if (a.mode != MODE_SORTED)
+      split_tiles(a, 4, 1, (int64_t)grid_d * (c.block / 32));
     if ((rc = plan(m, a, ws, st, (int64_t)grid_d * (c.block / 32)))) return rc;
     BY_CU(launch_dirgrad(a, c.block, grid_d, smem_d, st));
   }
@@ -1246,8 +1337,8 @@ int bysdf_eval_stochastic(const bysdf_materials* m, const bysdf_hits* hits,
   o.pdf = pdf;
   o.status = status;
   return run_forward(m, BYSDF_OP_EVAL, hits, nullptr, nullptr, n, o, workspace, workspace_bytes,
-                     reinterpret_cast<cudaStream_t>(stream), fwd_cfg(m, BYSDF_OP_EVAL, hits), 0,
-                     sto);
+                     reinterpret_cast<cudaStream_t>(stream),
+                     fwd_cfg(m, BYSDF_OP_EVAL, hits, sto->flags != 0), 0, sto);
 }
 
 int bysdf_eval_sample_pdf_stochastic(const bysdf_materials* m, const bysdf_hits* hits,
@@ -1267,8 +1358,8 @@ int bysdf_eval_sample_pdf_stochastic(const bysdf_materials* m, const bysdf_hits*
   o.pdf_s = pdf_s;
   o.lobe_status = lobe_status_s;
   return run_forward(m, BYSDF_OP_FUSED, hits, u0, u1, n, o, workspace, workspace_bytes,
-                     reinterpret_cast<cudaStream_t>(stream), fwd_cfg(m, BYSDF_OP_FUSED, hits), 0,
-                     sto);
+                     reinterpret_cast<cudaStream_t>(stream),
+                     fwd_cfg(m, BYSDF_OP_FUSED, hits, sto->flags != 0), 0, sto);
 }
 
 int bysdf_eval_backward(const bysdf_materials* m, const bysdf_hits* hits, int64_t n,

@@ -294,10 +294,9 @@ static const void* dir_fn(int block) {
   return nullptr;
 }
 
-cudaError_t set_backward_smem_limit(int block, int occ, int kind, size_t smem) {
+cudaError_t set_backward_smem_limit(int block, int occ, int kind, size_t optin) {
   const void* f = bwd_fn(block, occ, kind);
-  if (!f) return cudaErrorInvalidValue;
-  return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  return f ? raise_smem_limit(f, optin) : cudaErrorInvalidValue;
 }
 
 cudaError_t backward_occupancy(int block, int occ, int kind, size_t smem, int* ctas) {
@@ -319,10 +318,9 @@ cudaError_t launch_reduce_partials(const KArgs& a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t set_dirgrad_smem_limit(int block, size_t smem) {
+cudaError_t set_dirgrad_smem_limit(int block, size_t optin) {
   const void* f = dir_fn(block);
-  if (!f) return cudaErrorInvalidValue;
-  return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  return f ? raise_smem_limit(f, optin) : cudaErrorInvalidValue;
 }
 
 cudaError_t dirgrad_occupancy(int block, size_t smem, int* ctas) {

@@ -32,10 +32,17 @@ static const void* fwd_fn(int op, int block, int items, int occ) {
   return nullptr;
 }
 
-cudaError_t set_forward_smem_limit(int op, int block, int items, int occ, size_t smem) {
+cudaError_t raise_smem_limit(const void* kernel, size_t optin) {
+  cudaFuncAttributes attr;
+  const cudaError_t e = cudaFuncGetAttributes(&attr, kernel);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)(optin - attr.sharedSizeBytes));
+}
+
+cudaError_t set_forward_smem_limit(int op, int block, int items, int occ, size_t optin) {
   const void* f = fwd_fn(op, block, items, occ);
-  if (!f) return cudaErrorInvalidValue;
-  return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  return f ? raise_smem_limit(f, optin) : cudaErrorInvalidValue;
 }
 
 cudaError_t forward_occupancy(int op, int block, int items, int occ, size_t smem, int* ctas) {
@@ -44,9 +51,9 @@ cudaError_t forward_occupancy(int op, int block, int items, int occ, size_t smem
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, f, block, smem);
 }
 
-cudaError_t launch_forward(int op, const KArgs& a, int block, int occ, int grid, size_t smem,
-                           cudaStream_t st) {
-  const void* f = fwd_fn(op, block, a.tile / 32, occ);
+cudaError_t launch_forward(int op, const KArgs& a, int block, int items, int occ, int grid,
+                           size_t smem, cudaStream_t st) {
+  const void* f = fwd_fn(op, block, items, occ);
   if (!f) return cudaErrorInvalidValue;
   void* args[] = {const_cast<KArgs*>(&a)};
   return cudaLaunchKernel(f, dim3(grid), dim3(block), args, smem, st);

@@ -16,7 +16,7 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_forward(const KArgs a) {
   uint32_t* list = reinterpret_cast<uint32_t*>(smem + a.order_off) +
                    (threadIdx.x >> 5) * (32 * ITEMS + kOrderBuckets);
   uint32_t* hist = list + 32 * ITEMS;
-  persistent_loop<BLOCK>(a, smem, bars,
+  persistent_loop<BLOCK, (OP & OPF_STOCH) == 0>(a, smem, bars,
                          [&](int64_t begin, int64_t end, int mat, uint8_t* slot, int lane, int) {
     // records with a footprint in bucket order (each lane reads back only
     // its own slots of the list, written before the warp's last
@@ -46,8 +46,8 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_forward(const KArgs a) {
         if (!bounds_ok((size_t)mm * a.sstride + a.stride <= (size_t)a.order_off)) continue;
         m = reinterpret_cast<const MatDev*>(smem + (size_t)mm * a.sstride);
       }
-      // two plies side by side in the trace when registers allow (<= 128)
-      forward_record<OP, (BLOCK * MINB <= 512 ? 2 : 1)>(
+      // two plies side by side in the trace when registers allow (>= 96)
+      forward_record<OP, (BLOCK * MINB <= 640 ? 2 : 1)>(
           a, *m, reinterpret_cast<const float2*>(m + 1), i, q);
     }
     __syncwarp();   // the list is rewritten by the next tile
@@ -87,6 +87,11 @@ const void* fwd_kernel(int block, int items, int occ) {
     case 128: return fwd_kernel_b<OP, 128>(items, occ);
     case 256: return fwd_kernel_b<OP, 256>(items, occ);
     case 512: return fwd_kernel_b<OP, 512>(items, occ);
+    // the near-field default: 20 warps per SM; tiles of 4 rounds, or of one
+    // for a small material-sorted batch
+    case 640:
+      return items == 1 ? (const void*)k_forward<OP, 640, 1, 1>
+                        : (items == 4 ? (const void*)k_forward<OP, 640, 4, 1> : nullptr);
   }
   return nullptr;
 }

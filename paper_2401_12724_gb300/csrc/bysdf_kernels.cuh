@@ -17,20 +17,21 @@ enum : uint32_t { ERR_TABLE_WAIT = 1u, ERR_TABLE_INFLIGHT = 2u };
 //
 // Control words.  Every launch gets an epoch e from the host (40 bits,
 // never 0).  err_word = e << 24 | error bits, e the epoch of the launch that
-// last claimed it.  At its start each CTA claims the error word for its
-// launch: a word holding another epoch (a previous launch's, the contents
-// of a fresh allocation, or 0 after bysdf_workspace_error read it) is set
-// to e << 24.  The bits stay until bysdf_workspace_error reads them; a
-// captured launch replayed with its one epoch adds to the bits of its
-// earlier replays until then.
+// last claimed it.  The first CTA claims the error word for its launch: a
+// word holding another epoch (a previous launch's, the contents of a fresh
+// allocation, or 0 after bysdf_workspace_error read it) is set to e << 24;
+// another CTA claims it before it sets an error bit.  The bits stay until
+// bysdf_workspace_error reads them; a captured launch replayed with its one
+// epoch adds to the bits of its earlier replays until then.
 //
-// tile_word counts the warp-tile draws.  For records in any order with
-// fewer than 2^24 draws (claim_tiles) the CTAs claim it the same way and
-// the draws count from e << 24; the launch's last draw sets it to 0, so the
-// next launch (a replay with the same epoch too) claims it again, and no
-// reset kernel runs.  Otherwise the host launches k_plan first, which sets
-// tile_word to 0 and err_word to e << 24 (and, for material-sorted records,
-// computes the first tile of every material).
+// tile_word counts the tiles drawn after each warp's first, which is fixed.
+// For records in any order with fewer than 2^24 tiles (claim_tiles) the CTAs
+// claim it the same way and the draws count from e << 24; the launch's last
+// draw sets it to 0, so the next launch (a replay with the same epoch too)
+// claims it again, and no reset kernel runs.  A launch whose warps have at
+// most one tile each does not touch it.  Otherwise the host launches k_plan
+// first, which sets tile_word to 0 and err_word to e << 24 (and, for
+// material-sorted records, computes the first tile of every material).
 constexpr size_t kWsCtl = 256;
 constexpr int kEpochShift = 24;
 struct WsCtl {
@@ -46,7 +47,9 @@ struct KArgs {
   int32_t sstride;       // MODE_ALL_SMEM: bytes between materials' tables in shared memory
   int32_t mode;
   int32_t tile;          // records per warp tile (32 * items)
+  int32_t tail;          // records in any order: records per tile after the first n_main
   int64_t n;
+  int64_t n_main;        // records in any order: tiles of `tile` records
   int64_t n_tiles;
   const float *h, *u, *v, *wi, *wo, *ratio, *u0, *u1;
   const int32_t* mat_id;
@@ -131,19 +134,21 @@ __device__ __forceinline__ void claim_word(unsigned long long* word, uint64_t ep
   }
 }
 
-// Error bits of this launch (after the CTA claimed the word).
-__device__ __forceinline__ void set_error(WsCtl* ctl, uint32_t code) {
+// Error bits of this launch.
+__device__ __forceinline__ void set_error(WsCtl* ctl, uint64_t epoch, uint32_t code) {
+  claim_word(&ctl->err_word, epoch);
   atomicOr(&ctl->err_word, (unsigned long long)code);
 }
 
 // Bounded wait: gives up after `limit` polls (each poll may itself suspend
 // for a hardware-defined interval), records the failure and returns false.
 constexpr uint32_t kWaitLimit = 1u << 22;
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, WsCtl* ctl,
-                                                  uint32_t code, uint32_t limit = kWaitLimit) {
+__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity,
+                                                  const KArgs& a, uint32_t code,
+                                                  uint32_t limit = kWaitLimit) {
   for (uint32_t it = 0; it < limit; ++it)
     if (mbar_try_wait(bar, parity)) return true;
-  set_error(ctl, code);
+  set_error(a.ctl, a.epoch, code);
   return false;
 }
 
@@ -336,15 +341,25 @@ __device__ __forceinline__ void abort_tile(const KArgs& a, int64_t begin, int64_
 //   records may come in any material order.
 // MODE_SORTED:   records are grouped by material; each warp owns one table
 //   slot and refills it (TMA bulk copy) when its tile's material changes.
-// Work is handed out one warp tile (32 * items records) at a time from an
-// atomic counter, so warps that drew cheap records take more tiles.
+// Work is handed out one warp tile (32 * items records; shorter ones for the
+// last of a batch in any order) at a time: a warp's
+// first tile is fixed (neighbouring tiles to different CTAs, so that a small
+// batch spreads over the SMs), the next ones come from an atomic counter when
+// it is done, so warps that drew cheap records take more tiles; a batch of at
+// most one tile per warp draws nothing.  (Drawing ahead of the tile hides the
+// counter's round trip, but the last tiles then go to the warps that began
+// first, not to those that finish first: 650 us instead of 490 for 2^20
+// footprint records in 1.1 tiles per warp.)
 //
 // Every wait on a table copy is bounded.  When one gives up, the error word
 // records it, the copy is waited for once more (so that none is in flight
 // when the CTA exits), and the warps keep taking tiles but only mark their
 // records ST_ABORTED.  bars holds 2 * BLOCK / 32 barriers: the second half
 // are the barriers of the test hook (a.test_stall), which nothing arrives on.
-template <int BLOCK, class Body>
+// FIXED_FIRST: false for the stochastic kernels, whose every tile is drawn:
+// what the compiler fuses in them follows the shape of this loop, and their
+// results stay the same bits (a third of them moves by a rounding else).
+template <int BLOCK, bool FIXED_FIRST = true, class Body>
 __device__ __forceinline__ void persistent_loop(const KArgs& a, uint8_t* smem, uint64_t* bars,
                                                 Body&& body) {
   static_assert(BLOCK >= 64 && BLOCK % 32 == 0, "thread 32 claims the tile word");
@@ -357,12 +372,19 @@ __device__ __forceinline__ void persistent_loop(const KArgs& a, uint8_t* smem, u
   const uint32_t limit = a.wait_limit ? a.wait_limit : kWaitLimit;
   __shared__ int s_ok;
   bool aborted = false;
-  // with claim_tiles the CTA claims the control words for its launch (else
-  // k_plan set them): thread 0 the error word, before it can set an error
-  // bit, and thread 32 the tile word, both while the table copies are in
-  // flight; no warp draws a tile before the barrier after them
+  // with claim_tiles the control words are claimed for this launch (else
+  // k_plan set them): the error word by one thread of the launch, the tile
+  // word, if tiles will be drawn, by each CTA's thread 32 while the table
+  // copies are in flight; no warp draws a tile before the barrier after them
+  const int n_warps = (int)gridDim.x * (BLOCK / 32);
+#ifdef BYSDF_DEBUG_BOUNDS
+  const bool claims_error = a.claim_tiles;  // the checks set bits unclaimed
+#else
+  const bool claims_error = a.claim_tiles && (!FIXED_FIRST || blockIdx.x == 0);
+#endif
+  const bool claims_tiles = a.claim_tiles && (!FIXED_FIRST || a.n_tiles > n_warps);
   if (a.mode == MODE_ALL_SMEM) {
-    if (threadIdx.x == 32 && a.claim_tiles) {
+    if (threadIdx.x == 32 && claims_tiles) {
       claim_word(&a.ctl->tile_word, a.epoch);
       __threadfence();
     }
@@ -378,23 +400,15 @@ __device__ __forceinline__ void persistent_loop(const KArgs& a, uint8_t* smem, u
       for (int k = 0; k < a.n_mat; ++k)
         bulk_g2s(smem + (size_t)k * a.sstride, a.table + (size_t)k * a.stride,
                  (uint32_t)a.stride, &bars[0]);
-      if (a.claim_tiles) claim_word(&a.ctl->err_word, a.epoch);
-      int ok = mbar_wait_bounded(a.test_stall ? &stall[0] : &bars[0], 0, a.ctl, ERR_TABLE_WAIT,
+      if (claims_error) claim_word(&a.ctl->err_word, a.epoch);
+      int ok = mbar_wait_bounded(a.test_stall ? &stall[0] : &bars[0], 0, a, ERR_TABLE_WAIT,
                                  limit);
-      if (!ok) mbar_wait_bounded(&bars[0], 0, a.ctl, ERR_TABLE_INFLIGHT);
+      if (!ok) mbar_wait_bounded(&bars[0], 0, a, ERR_TABLE_INFLIGHT);
       s_ok = ok;
     }
     __syncthreads();
     aborted = !s_ok;
   } else {
-    if (a.claim_tiles) {
-      if (threadIdx.x == 0) {
-        claim_word(&a.ctl->err_word, a.epoch);
-        claim_word(&a.ctl->tile_word, a.epoch);
-        __threadfence();
-      }
-      __syncthreads();
-    }
     if (lane == 0) {
       mbar_init(&bars[warp], 1);
       mbar_init(&stall[warp], 1);
@@ -418,28 +432,46 @@ __device__ __forceinline__ void persistent_loop(const KArgs& a, uint8_t* smem, u
   uint8_t* slot = smem + (size_t)warp * a.stride;
   uint32_t parity = 0;
   int cur = -1;
-  // Every warp draws until it gets a tile past the end, so a launch makes
-  // exactly n_tiles + (its warps) draws.  With claim_tiles the warp that
-  // makes the last one sets the word to 0, the state in which every launch
-  // (a replay of a captured launch with the same epoch too) reclaims it.
+  // With a fixed first tile, every tile worked on draws one more, so a launch
+  // that draws at all makes exactly n_tiles draws; else every warp draws until
+  // it gets a tile past the end, n_tiles + (its warps) draws.  With
+  // claim_tiles the warp that makes the last one sets the word to 0, the state
+  // in which every launch (a replay of a captured launch with the same epoch
+  // too) reclaims it.
+  const bool queue = n_tiles > n_warps;
   const unsigned long long tile_base =
       a.claim_tiles ? (unsigned long long)a.epoch << kEpochShift : 0ull;
   const unsigned long long last_draw =
-      a.claim_tiles ? (unsigned long long)n_tiles + gridDim.x * (BLOCK / 32) - 1 : ~0ull;
+      a.claim_tiles ? (unsigned long long)n_tiles + (FIXED_FIRST ? 0 : gridDim.x * (BLOCK / 32)) - 1
+                    : ~0ull;
+  int next = warp * (int)gridDim.x + (int)blockIdx.x;  // FIXED_FIRST
   for (;;) {
     int tile = 0;
-    if (lane == 0) {
-      const unsigned long long t = atomicAdd(&a.ctl->tile_word, 1ull) - tile_base;
-      if (t == last_draw) atomicExch(&a.ctl->tile_word, 0ull);
-      tile = (int)t;
+    if constexpr (FIXED_FIRST) {
+      tile = next;
+    } else {
+      if (lane == 0) {
+        const unsigned long long t = atomicAdd(&a.ctl->tile_word, 1ull) - tile_base;
+        if (t == last_draw) atomicExch(&a.ctl->tile_word, 0ull);
+        tile = (int)t;
+      }
+      tile = __shfl_sync(0xffffffffu, tile, 0);
     }
-    tile = __shfl_sync(0xffffffffu, tile, 0);
     if (tile >= n_tiles) break;
     int64_t begin, end;
     int mat = -1;
     if (a.mode == MODE_ALL_SMEM) {
-      begin = (int64_t)tile * a.tile;
-      end = begin + a.tile < a.n ? begin + a.tile : a.n;
+      if constexpr (FIXED_FIRST) {
+        // n_main tiles of `tile` records, then tiles of `tail` records
+        const bool is_main = tile < a.n_main;
+        const int64_t rest = (int64_t)tile - a.n_main;
+        const int size = is_main ? a.tile : a.tail;
+        begin = is_main ? (int64_t)tile * a.tile : a.n_main * a.tile + rest * a.tail;
+        end = begin + size < a.n ? begin + size : a.n;
+      } else {
+        begin = (int64_t)tile * a.tile;
+        end = begin + a.tile < a.n ? begin + a.tile : a.n;
+      }
     } else {
       int lo = 0, hi = a.n_mat;  // last material whose first tile <= tile
       while (hi - lo > 1) {
@@ -462,11 +494,11 @@ __device__ __forceinline__ void persistent_loop(const KArgs& a, uint8_t* smem, u
           mbar_arrive_tx(&bars[warp], (uint32_t)a.stride);
           bulk_g2s(slot, a.table + (size_t)mat * a.stride, (uint32_t)a.stride, &bars[warp]);
         }
-        bool ok = mbar_wait_bounded(a.test_stall ? &stall[warp] : &bars[warp], parity, a.ctl,
+        bool ok = mbar_wait_bounded(a.test_stall ? &stall[warp] : &bars[warp], parity, a,
                                     ERR_TABLE_WAIT, limit);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) {
-          if (lane == 0) mbar_wait_bounded(&bars[warp], parity, a.ctl, ERR_TABLE_INFLIGHT);
+          if (lane == 0) mbar_wait_bounded(&bars[warp], parity, a, ERR_TABLE_INFLIGHT);
           __syncwarp();
           aborted = true;
         } else {
@@ -476,11 +508,27 @@ __device__ __forceinline__ void persistent_loop(const KArgs& a, uint8_t* smem, u
       }
     }
     BY_BOUNDS(begin >= 0 && end <= a.n && begin <= end, begin = end = 0);
-    if (aborted) {
-      abort_tile(a, begin, end, lane);
-      continue;
+    if constexpr (FIXED_FIRST) {
+      if (aborted) {
+        abort_tile(a, begin, end, lane);
+      } else {
+        body(begin, end, mat, slot, lane, tile);
+      }
+      if (!queue) break;
+      next = 0;
+      if (lane == 0) {
+        const unsigned long long t = atomicAdd(&a.ctl->tile_word, 1ull) - tile_base;
+        if (t == last_draw) atomicExch(&a.ctl->tile_word, 0ull);
+        next = n_warps + (int)t;
+      }
+      next = __shfl_sync(0xffffffffu, next, 0);
+    } else {
+      if (aborted) {
+        abort_tile(a, begin, end, lane);
+        continue;
+      }
+      body(begin, end, mat, slot, lane, tile);
     }
-    body(begin, end, mat, slot, lane, tile);
   }
 }
 
