@@ -2,6 +2,7 @@
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 import os
 import threading
 
@@ -9,6 +10,8 @@ from . import build as _build
 
 _lock = threading.Lock()
 _lib = None
+# the native call path of api.py (csrc/bysdf_torch.cpp), set by load()
+calls = None
 
 
 class MaterialDesc(C.Structure):
@@ -119,7 +122,7 @@ def lib_path() -> str:
 def load(build_if_missing: bool = True):
     """Load libbysdf.so (building it first if asked).  There is no fallback:
     without the library every call raises."""
-    global _lib
+    global _lib, calls
     with _lock:
         if _lib is not None:
             return _lib
@@ -133,6 +136,12 @@ def load(build_if_missing: bool = True):
             f = getattr(L, name)
             f.restype = res
             f.argtypes = args
+        if os.path.exists(_build.BINDING_PATH):
+            spec = importlib.util.spec_from_file_location("_bysdf_torch", _build.BINDING_PATH)
+            m = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(m)
+            m.bind({name: C.cast(getattr(L, name), C.c_void_p).value for name, _, _ in SYMBOLS})
+            calls = m
         _lib = L
         return _lib
 

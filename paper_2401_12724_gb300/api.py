@@ -2,6 +2,9 @@
 
 Argument marshalling only: tensors are passed to the C ABI as raw device
 pointers and every step of the BYSDF runs in the library's CUDA kernels.
+Plain calls (torch tensors on the GPU, outputs allocated by the call) go
+through the native call path (csrc/bysdf_torch.cpp); it leaves every other
+call to the code here.
 Records are a dict of CUDA tensors: h, u, v (n,), wi, wo (3, n) float32,
 optional mat_id (n,) int32, ratio (n,) float32, seg_offsets (n_mat + 1,)
 int64.  Outputs are allocated here with torch (device memory is plumbing).
@@ -91,6 +94,8 @@ class Materials:
         return self._ws
 
     def set_params(self, params: torch.Tensor, stream=None):
+        if _call("set_params", "bysdf_set_params", 8, self, params, stream=stream) is None:
+            return
         p = params.detach().to(device=self.device, dtype=torch.float32).contiguous()
         assert p.shape == (self.n_mat, 8)
         N.check(self.lib.bysdf_set_params(self.handle, _ptr(p), _stream(stream)), "bysdf_set_params")
@@ -103,6 +108,9 @@ class Materials:
 
     def set_params_ext(self, params: torch.Tensor, stream=None):
         """The 15 parameters of the extended set (bysdf_set_params_ext)."""
+        if _call("set_params", "bysdf_set_params_ext", N.NPARAM_EXT, self, params,
+                 stream=stream) is None:
+            return
         p = params.detach().to(device=self.device, dtype=torch.float32).contiguous()
         assert p.shape == (self.n_mat, N.NPARAM_EXT)
         N.check(self.lib.bysdf_set_params_ext(self.handle, _ptr(p), _stream(stream)),
@@ -168,12 +176,27 @@ def _n(rec) -> int:
     return int(rec["h"].shape[0])
 
 
+def _call(name, what, *args, stream=None):
+    """The native call path, or NotImplemented where it does not take the call."""
+    if N.calls is None:
+        return NotImplemented
+    r = getattr(N.calls, name)(*args, None if stream is None else _stream(stream))
+    if type(r) is int:
+        N.check(r, what)
+    return r
+
+
 def _empty(shape, dtype, dev):
     return torch.empty(shape, dtype=dtype, device=dev)
 
 
 def eval(mats: Materials, rec: dict, with_pdf: bool = True, stream=None, out=None):
     """f |wo.n| (3, n), pdf (n,) and status (n,) uint8."""
+    if not out:
+        r = _call("forward", "bysdf_eval", N.OP_EVAL, mats, rec, None, None, bool(with_pdf),
+                  stream=stream)
+        if r is not NotImplemented:
+            return r
     n = _n(rec)
     dev = rec["h"].device
     f = out["f"] if out else _empty((3, n), torch.float32, dev)
@@ -187,6 +210,10 @@ def eval(mats: Materials, rec: dict, with_pdf: bool = True, stream=None, out=Non
 
 def sample(mats: Materials, rec: dict, u0=None, u1=None, stream=None, out=None):
     """wo (3, n), weight (3, n), pdf (n,), lobe << 4 | status (n,)."""
+    if not out:
+        r = _call("forward", "bysdf_sample", N.OP_SAMPLE, mats, rec, u0, u1, True, stream=stream)
+        if r is not NotImplemented:
+            return r
     n = _n(rec)
     dev = rec["h"].device
     u0 = rec["u0"] if u0 is None else u0
@@ -204,6 +231,10 @@ def sample(mats: Materials, rec: dict, u0=None, u1=None, stream=None, out=None):
 
 
 def pdf(mats: Materials, rec: dict, stream=None, out=None):
+    if not out:
+        r = _call("forward", "bysdf_pdf", N.OP_PDF, mats, rec, None, None, True, stream=stream)
+        if r is not NotImplemented:
+            return r
     n = _n(rec)
     dev = rec["h"].device
     p = out["pdf"] if out else _empty((n,), torch.float32, dev)
@@ -223,6 +254,11 @@ def alloc_fused(n: int, dev) -> dict:
 
 def eval_sample_pdf(mats: Materials, rec: dict, u0=None, u1=None, stream=None, out=None) -> dict:
     """Fused eval + pdf at rec['wo'] and a sample from (u0, u1)."""
+    if out is None:
+        r = _call("forward", "bysdf_eval_sample_pdf", N.OP_FUSED, mats, rec, u0, u1, True,
+                  stream=stream)
+        if r is not NotImplemented:
+            return r
     n = _n(rec)
     o = out if out is not None else alloc_fused(n, rec["h"].device)
     u0 = rec["u0"] if u0 is None else u0
@@ -310,6 +346,11 @@ def trace_yarns(yarns: torch.Tensor, rays: dict, light, stream=None, out=None) -
 def eval_backward(mats: Materials, rec: dict, grad_f: torch.Tensor, deterministic: bool = False,
                   stream=None, out=None) -> torch.Tensor:
     """d(sum grad_f * f) / d params, shape (n_mat, 8)."""
+    if out is None:
+        r = _call("backward", "bysdf_eval_backward", 0, mats, rec, grad_f, None, False,
+                  bool(deterministic), stream=stream)
+        if r is not NotImplemented:
+            return r
     n = _n(rec)
     g = out if out is not None else _empty((mats.n_mat, 8), torch.float32, rec["h"].device)
     gf = grad_f.contiguous()
@@ -325,6 +366,10 @@ def eval_l2_backward(mats: Materials, rec: dict, target: torch.Tensor, weight=No
     """Forward, L2 loss against target (3, n) and its parameter gradient in
     one pass (bysdf_eval_l2_backward): returns grad (n_mat, 8), per-material
     loss (n_mat,) and f (3, n) (None unless with_f)."""
+    r = _call("backward", "bysdf_eval_l2_backward", 2, mats, rec, target, weight, bool(with_f),
+              bool(deterministic), stream=stream)
+    if r is not NotImplemented:
+        return r
     n = _n(rec)
     dev = rec["h"].device
     g = _empty((mats.n_mat, 8), torch.float32, dev)
@@ -343,6 +388,10 @@ def eval_backward_ext(mats: Materials, rec: dict, grad_f: torch.Tensor,
                       deterministic: bool = False, dirs: bool = False, stream=None):
     """d(sum grad_f * f) / d params for the 15-column extended set, and with
     dirs=True the per-record products grad_f . df/dwi and . df/dwo (3, n)."""
+    r = _call("backward", "bysdf_eval_backward_ext", 1, mats, rec, grad_f, None, bool(dirs),
+              bool(deterministic), stream=stream)
+    if r is not NotImplemented:
+        return r
     n = _n(rec)
     dev = rec["h"].device
     g = _empty((mats.n_mat, N.NPARAM_EXT), torch.float32, dev)

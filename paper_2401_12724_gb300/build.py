@@ -1,4 +1,5 @@
-"""Builds libbysdf.so in-tree with nvcc for sm_103a (no CMake, no torch)."""
+"""Builds libbysdf.so in-tree with nvcc for sm_103a (no CMake, no torch), and
+the call path of api.py against torch's headers (one host translation unit)."""
 from __future__ import annotations
 
 import os
@@ -18,6 +19,9 @@ LIB_PATH = os.path.join(PKG, "libbysdf.so")
 # a separate library, built on demand by the tests that use it.
 BOUNDS_BUILD_DIR = os.path.join(BUILD_DIR, "bounds")
 BOUNDS_LIB_PATH = os.path.join(PKG, "libbysdf_bounds.so")
+# The native call path of api.py (csrc/bysdf_torch.cpp); both libraries use it.
+BINDING_SRC = os.path.join(CSRC, "bysdf_torch.cpp")
+BINDING_PATH = os.path.join(PKG, "_bysdf_torch.so")
 SOURCES = ["bysdf_api.cu", "bysdf_fwd.cu", "bysdf_fwd_eval.cu", "bysdf_fwd_sample.cu",
            "bysdf_fwd_pdf.cu", "bysdf_fwd_fused.cu", "bysdf_fwd_stoch.cu", "bysdf_bwd.cu",
            "bysdf_trace.cu"]
@@ -49,11 +53,35 @@ def _deps():
     return [os.path.join(CSRC, s) for s in SOURCES] + hdrs + [os.path.join(INCLUDE, "bysdf.h")]
 
 
-def _stale(lib: str) -> bool:
+def _stale(lib: str, deps=None) -> bool:
     if not os.path.exists(lib):
         return True
     t = os.path.getmtime(lib)
-    return any(os.path.getmtime(p) > t for p in _deps())
+    return any(os.path.getmtime(p) > t for p in deps or _deps())
+
+
+def _build_binding(force: bool) -> None:
+    if not force and not _stale(BINDING_PATH,
+                                [BINDING_SRC, os.path.join(INCLUDE, "bysdf.h")]):
+        return
+    import sysconfig
+
+    import torch
+    from torch.utils import cpp_extension as X
+
+    inc = [*X.include_paths(), sysconfig.get_paths()["include"],
+           os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include")]
+    tmp = BINDING_PATH + f".tmp{os.getpid()}"
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-w",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           *(f"-I{p}" for p in [INCLUDE, *inc]), BINDING_SRC, "-o", tmp]
+    for d in X.library_paths():
+        cmd += [f"-L{d}", f"-Wl,-rpath,{d}"]
+    cmd += ["-ltorch_python", "-ltorch", "-ltorch_cpu", "-ltorch_cuda", "-lc10", "-lc10_cuda"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"g++ failed for bysdf_torch.cpp:\n{r.stderr}")
+    os.replace(tmp, BINDING_PATH)
 
 
 def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False,
@@ -65,6 +93,7 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False,
     defs = ["-DBYSDF_DEBUG_BOUNDS"] if bounds else []
     with _lock:
         if not force and not _stale(lib):
+            _build_binding(False)
             return lib
         os.makedirs(bdir, exist_ok=True)
         nvcc = _nvcc()
@@ -81,8 +110,10 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False,
                 sys.stderr.write(r.stderr)
             return obj
 
-        with ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
+        with ThreadPoolExecutor(max_workers=len(SOURCES) + 1) as ex:
+            binding = ex.submit(_build_binding, force and not bounds)
             objs = list(ex.map(compile_one, SOURCES))
+            binding.result()
         tmp = lib + f".tmp{os.getpid()}"
         cmd = [nvcc, *ARCH, "-shared", "-cudart", "static", "-o", tmp, *objs]
         r = subprocess.run(cmd, capture_output=True, text=True)

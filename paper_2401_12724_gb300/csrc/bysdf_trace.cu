@@ -15,6 +15,9 @@
 // distance (no cancellation between terms of the camera distance squared).
 // The culling only skips pieces that no ray of the warp can hit: the result
 // is that of testing every piece.
+#include <mutex>
+#include <vector>
+
 #include "bysdf_launch.h"
 
 namespace bysdf {
@@ -294,19 +297,38 @@ cudaError_t launch_trace_yarns(const bysdf_yarn* yarns, int n_yarns, const Trace
   const int n_grp = (n_yarns + kGroupPieces - 1) / kGroupPieces;
   const size_t smem = sizeof(PieceS) * (size_t)n_yarns + sizeof(float4) * (size_t)n_grp +
                       sizeof(int32_t) * (size_t)n_yarns;
-  cudaError_t e;
-  if (smem > 48 * 1024) {
-    e = cudaFuncSetAttribute(k_trace_yarns, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  // one resident wave: every CTA stages the pieces once
+  // one resident wave: every CTA stages the pieces once.  What the device
+  // holds is looked up once per device and size (host time of every call)
+  struct Entry {
+    int dev, sms, per_sm;
+    size_t smem;
+  };
+  static std::mutex mu;
+  static std::vector<Entry> seen;
   int dev = 0, sms = 0, per_sm = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
-      (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
-      (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_trace_yarns, 256, smem)) !=
-          cudaSuccess)
-    return e;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    for (const Entry& x : seen)
+      if (x.dev == dev && x.smem == smem) {
+        sms = x.sms;
+        per_sm = x.per_sm;
+      }
+    if (sms == 0) {
+      int optin = 0;
+      if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) !=
+              cudaSuccess ||
+          (smem > 48 * 1024 &&
+           (e = raise_smem_limit((const void*)k_trace_yarns, (size_t)optin)) != cudaSuccess) ||
+          (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+          (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_trace_yarns, 256, smem)) !=
+              cudaSuccess)
+        return e;
+      if (seen.size() >= 256) seen.clear();  // sizes come from the caller
+      seen.push_back({dev, sms, per_sm, smem});
+    }
+  }
   if (per_sm > 0 && grid > sms * per_sm) grid = sms * per_sm;
   k_trace_yarns<<<grid, 256, smem, st>>>(yarns, n_yarns, a);
   return cudaGetLastError();
