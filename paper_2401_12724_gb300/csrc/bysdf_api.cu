@@ -1317,12 +1317,7 @@ int bysdf_trace_yarns(const bysdf_yarn* yarns, int32_t n_yarns, const bysdf_rays
   a.t_hit = t_hit;
   a.mat_id = mat_id;
   a.yarn_id = yarn_id;
-  int dev = 0, sms = 0;
-  BY_CU(cudaGetDevice(&dev));
-  BY_CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int64_t blocks = (n + 255) / 256;
-  const int grid = (int)std::min<int64_t>(blocks, (int64_t)sms * 8);
-  BY_CU(launch_trace_yarns(yarns, n_yarns, a, grid, reinterpret_cast<cudaStream_t>(stream)));
+  BY_CU(launch_trace_yarns(yarns, n_yarns, a, reinterpret_cast<cudaStream_t>(stream)));
   return BYSDF_OK;
 }
 

@@ -18,7 +18,7 @@ struct TraceArgs {
 };
 constexpr int kMaxYarnPieces = 2048;  // 64 bytes each in shared memory
 cudaError_t launch_trace_yarns(const bysdf_yarn* yarns, int n_yarns, const TraceArgs& a,
-                               int grid, cudaStream_t st);
+                               cudaStream_t st);
 
 // op: OPF_* bit set (EVAL, SAMPLE, PDF, EVAL|SAMPLE).  Returns the launch error.
 cudaError_t launch_forward(int op, const KArgs& a, int block, int items, int occ, int grid,
