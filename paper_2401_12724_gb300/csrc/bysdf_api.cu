@@ -658,6 +658,12 @@ int run_forward(const bysdf_materials* m, int op, const bysdf_hits* h, const flo
       }
     } else if (a.n_tiles < warps) {
       items = tile = 1;
+    } else if (!m->cfg_set[op] && !h->ratio && !(bits & OPF_STOCH) && rounds < 16 * warps) {
+      // sorted near-field records, a few tiles per warp: shorter ones end
+      // together, more of them cost draws and table copies (fused: 5 rounds a
+      // warp 65.3 us in tiles of 4, 56.5 of 2, 58.4 of 1; 13 rounds 135, 129,
+      // 137; 18 rounds 177, 178, 191; 41 rounds 370, 376, 404)
+      tile = 2;
     }
     if (items != c.items) {
       c.items = items;
