@@ -126,7 +126,7 @@ struct Planes {
 
 }  // namespace
 
-// Bound by instruction issue (about 1000 warp instructions per 32 rays) and
+// Bound by instruction issue (1,110 warp instructions per 32 rays) and
 // the latency of the culling chain.  One CTA of 768 threads (24 warps, up to 85
 // registers) per SM shares one copy of the pieces: CTAs of 256 held up to three
 // copies, and 2048 pieces (140 KB) left room for one of 8 warps.  2048 x 2048
