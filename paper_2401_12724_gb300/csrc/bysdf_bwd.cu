@@ -296,7 +296,7 @@ static const void* dir_fn(int block) {
 
 cudaError_t set_backward_smem_limit(int block, int occ, int kind, size_t optin) {
   const void* f = bwd_fn(block, occ, kind);
-  return f ? raise_smem_limit(f, optin) : cudaErrorInvalidValue;
+  return f ? raise_smem_limit(f, optin, optin) : cudaErrorInvalidValue;
 }
 
 cudaError_t backward_occupancy(int block, int occ, int kind, size_t smem, int* ctas) {
@@ -320,7 +320,7 @@ cudaError_t launch_reduce_partials(const KArgs& a, cudaStream_t st) {
 
 cudaError_t set_dirgrad_smem_limit(int block, size_t optin) {
   const void* f = dir_fn(block);
-  return f ? raise_smem_limit(f, optin) : cudaErrorInvalidValue;
+  return f ? raise_smem_limit(f, optin, optin) : cudaErrorInvalidValue;
 }
 
 cudaError_t dirgrad_occupancy(int block, size_t smem, int* ctas) {

@@ -32,17 +32,18 @@ static const void* fwd_fn(int op, int block, int items, int occ) {
   return nullptr;
 }
 
-cudaError_t raise_smem_limit(const void* kernel, size_t optin) {
+cudaError_t raise_smem_limit(const void* kernel, size_t smem, size_t optin) {
   cudaFuncAttributes attr;
   const cudaError_t e = cudaFuncGetAttributes(&attr, kernel);
   if (e != cudaSuccess) return e;
+  if (attr.sharedSizeBytes + smem <= 48 * 1024) return cudaSuccess;
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)(optin - attr.sharedSizeBytes));
 }
 
 cudaError_t set_forward_smem_limit(int op, int block, int items, int occ, size_t optin) {
   const void* f = fwd_fn(op, block, items, occ);
-  return f ? raise_smem_limit(f, optin) : cudaErrorInvalidValue;
+  return f ? raise_smem_limit(f, optin, optin) : cudaErrorInvalidValue;
 }
 
 cudaError_t forward_occupancy(int op, int block, int items, int occ, size_t smem, int* ctas) {

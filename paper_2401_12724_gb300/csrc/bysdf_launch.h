@@ -30,8 +30,9 @@ cudaError_t launch_plain(int op, const KArgs& a, int mat, int64_t begin, int64_t
 cudaError_t launch_backward(const KArgs& a, int block, int occ, int kind, int grid, size_t smem,
                             cudaStream_t st);
 // Raises a kernel's dynamic shared-memory limit to what the device's opt-in
-// maximum leaves beside its static shared memory.
-cudaError_t raise_smem_limit(const void* kernel, size_t optin);
+// maximum leaves beside its static shared memory, where `smem` dynamic bytes
+// and the static ones together pass the 48 KB that need no opt-in.
+cudaError_t raise_smem_limit(const void* kernel, size_t smem, size_t optin);
 cudaError_t launch_reduce_partials(const KArgs& a, cudaStream_t st);
 cudaError_t set_forward_smem_limit(int op, int block, int items, int occ, size_t optin);
 cudaError_t set_backward_smem_limit(int block, int occ, int kind, size_t optin);

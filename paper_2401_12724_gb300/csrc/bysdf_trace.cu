@@ -404,16 +404,17 @@ cudaError_t launch_trace_yarns(const bysdf_yarn* yarns, int n_yarns, const Trace
       int optin = 0;
       if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) !=
               cudaSuccess ||
-          (smem > 48 * 1024 && (e = raise_smem_limit(kernel, (size_t)optin)) != cudaSuccess) ||
+          (e = raise_smem_limit(kernel, smem, (size_t)optin)) != cudaSuccess ||
           (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, smem)) !=
               cudaSuccess)
         return e;
+      if (per_sm < 1) return cudaErrorInvalidConfiguration;
       if (seen.size() >= 256) seen.clear();  // sizes come from the caller
       seen.push_back({dev, block, per_sm, smem});
     }
   }
   const int64_t ctas = (std::min(a.n, kMaxLaunch) + block - 1) / block;
-  const int grid = (int)std::min<int64_t>(ctas, (int64_t)sms * std::max(per_sm, 1));
+  const int grid = (int)std::min<int64_t>(ctas, (int64_t)sms * per_sm);
   for (int64_t at = 0; at < a.n; at += kMaxLaunch) {
     Planes p;
     const float* in[] = {a.o, a.d, a.o1, a.d1, a.o2, a.d2};
