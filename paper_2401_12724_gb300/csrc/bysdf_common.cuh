@@ -38,8 +38,10 @@ struct alignas(16) MatDev {
 static_assert(sizeof(MatDev) == 256, "MatDev must be 256 bytes");
 
 // Fiber migration map k >= 1 (Sec. 3.5): a 32-byte header, then T texels.
-// Map 0 is the regular ring whose constants live in MatDev.
-struct alignas(16) MigMap {
+// Map 0 is the regular ring whose constants live in MatDev.  The header lies
+// behind any number of texels, so it is aligned like one: an odd count leaves
+// no more than 8 bytes.
+struct MigMap {
   float m_over_2pi;     // M_k / (2 pi)
   float kf_hi, kf_lo;   // fiber phase rate in map periods per length, split
   float dkf;            // d kf / d alpha_f
@@ -48,6 +50,8 @@ struct alignas(16) MigMap {
   float aux;            // map 1 only: low part of 1 / segment length
 };
 static_assert(sizeof(MigMap) == 32, "MigMap must be 32 bytes");
+static_assert(sizeof(MatDev) % alignof(MigMap) == 0 && sizeof(float2) % alignof(MigMap) == 0,
+              "a MigMap lies behind MatDev and any number of texels");
 
 // Bytes of one material: header, map 0, K_m - 1 migration maps, and (when
 // migrating) the map index of each of 256 consecutive segments.
