@@ -549,11 +549,12 @@ void split_tiles(KArgs& a, int items, int tail_items, int64_t warps) {
   a.n_tiles = a.n_main + (rest + a.tail - 1) / a.tail;
 }
 
-// Resident CTAs per SM of a launch shape, with its kernel's shared-memory
-// limit raised (to the device's maximum, whatever the shape: a smaller table
-// must not lower it for a larger one).  Both are host time that every call
-// would pay, so they are looked up once per table and shape.  code: the op
-// bits, or kShapeBackward + kind, or kShapeDirgrad.
+// Resident CTAs per SM of a launch shape (0: none fits), with its kernel's
+// shared-memory limit raised where the shape needs it (to the device's maximum,
+// whatever the shape: a smaller table must not lower it for a larger one).
+// Both are host time that every call would pay, so they are looked up once per
+// table and shape.  code: the op bits, or kShapeBackward + kind, or
+// kShapeDirgrad.
 constexpr int kShapeBackward = 0x100, kShapeDirgrad = 0x200;
 cudaError_t cached_shape(const bysdf_materials* m, int code, int block, int items, int occ,
                          size_t smem, int* ctas) {
@@ -563,17 +564,16 @@ cudaError_t cached_shape(const bysdf_materials* m, int code, int block, int item
       *ctas = e.ctas;
       return cudaSuccess;
     }
-  const bool raise = smem > 48 * 1024;
   cudaError_t err = cudaSuccess;
   if (code == kShapeDirgrad) {
-    if (raise) err = set_dirgrad_smem_limit(block, m->smem_optin);
+    err = set_dirgrad_smem_limit(block, smem, m->smem_optin);
     if (err == cudaSuccess) err = dirgrad_occupancy(block, smem, ctas);
   } else if (code & kShapeBackward) {
     const int kind = code - kShapeBackward;
-    if (raise) err = set_backward_smem_limit(block, occ, kind, m->smem_optin);
+    err = set_backward_smem_limit(block, occ, kind, smem, m->smem_optin);
     if (err == cudaSuccess) err = backward_occupancy(block, occ, kind, smem, ctas);
   } else {
-    if (raise) err = set_forward_smem_limit(code, block, items, occ, m->smem_optin);
+    err = set_forward_smem_limit(code, block, items, occ, smem, m->smem_optin);
     if (err == cudaSuccess) err = forward_occupancy(code, block, items, occ, smem, ctas);
   }
   if (err == cudaSuccess) m->occ_cache.push_back({code, block, items, occ, smem, *ctas});
@@ -661,6 +661,8 @@ int run_forward(const bysdf_materials* m, int op, const bysdf_hits* h, const flo
   if ((size_t)a.order_off + (size_t)(c.block / 32) * order_bytes(c.items) > m->smem_optin)
     return fail(BYSDF_E_UNSUPPORTED, "material table too large for shared memory");
   BY_CU(shape(c.items));
+  // beside the kernel's static shared memory
+  if (occ < 1) return fail(BYSDF_E_UNSUPPORTED, "material table too large for shared memory");
   const int64_t warps = (int64_t)grid_for(m, c, occ) * (c.block / 32);
   if (a.mode != MODE_SORTED && !h->ratio && !(bits & OPF_STOCH)) {
     split_tiles(a, c.items, 1, warps);
@@ -786,6 +788,7 @@ int run_backward(const bysdf_materials* m, const bysdf_hits* h, int64_t n, const
   if (smem > m->smem_optin) return fail(BYSDF_E_UNSUPPORTED, "material table too large for shared memory");
   int occ = 0;
   BY_CU(cached_shape(m, kShapeBackward + kind, c.block, 0, c.occupancy, smem, &occ));
+  if (occ < 1) return fail(BYSDF_E_UNSUPPORTED, "material table too large for shared memory");
   if (!deterministic) BY_CU(cudaMemsetAsync(grad_params, 0, sizeof(float) * ng * m->n_mat, st));
   const int grid = grid_for(m, c, occ);
   const int64_t warps = (int64_t)grid * (c.block / 32);

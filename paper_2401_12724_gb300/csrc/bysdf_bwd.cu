@@ -294,9 +294,9 @@ static const void* dir_fn(int block) {
   return nullptr;
 }
 
-cudaError_t set_backward_smem_limit(int block, int occ, int kind, size_t optin) {
+cudaError_t set_backward_smem_limit(int block, int occ, int kind, size_t smem, size_t optin) {
   const void* f = bwd_fn(block, occ, kind);
-  return f ? raise_smem_limit(f, optin, optin) : cudaErrorInvalidValue;
+  return f ? raise_smem_limit(f, smem, optin) : cudaErrorInvalidValue;
 }
 
 cudaError_t backward_occupancy(int block, int occ, int kind, size_t smem, int* ctas) {
@@ -318,9 +318,9 @@ cudaError_t launch_reduce_partials(const KArgs& a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t set_dirgrad_smem_limit(int block, size_t optin) {
+cudaError_t set_dirgrad_smem_limit(int block, size_t smem, size_t optin) {
   const void* f = dir_fn(block);
-  return f ? raise_smem_limit(f, optin, optin) : cudaErrorInvalidValue;
+  return f ? raise_smem_limit(f, smem, optin) : cudaErrorInvalidValue;
 }
 
 cudaError_t dirgrad_occupancy(int block, size_t smem, int* ctas) {

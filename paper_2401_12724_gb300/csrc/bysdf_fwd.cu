@@ -41,9 +41,10 @@ cudaError_t raise_smem_limit(const void* kernel, size_t smem, size_t optin) {
                               (int)(optin - attr.sharedSizeBytes));
 }
 
-cudaError_t set_forward_smem_limit(int op, int block, int items, int occ, size_t optin) {
+cudaError_t set_forward_smem_limit(int op, int block, int items, int occ, size_t smem,
+                                   size_t optin) {
   const void* f = fwd_fn(op, block, items, occ);
-  return f ? raise_smem_limit(f, optin, optin) : cudaErrorInvalidValue;
+  return f ? raise_smem_limit(f, smem, optin) : cudaErrorInvalidValue;
 }
 
 cudaError_t forward_occupancy(int op, int block, int items, int occ, size_t smem, int* ctas) {

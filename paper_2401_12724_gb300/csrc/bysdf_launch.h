@@ -34,12 +34,13 @@ cudaError_t launch_backward(const KArgs& a, int block, int occ, int kind, int gr
 // and the static ones together pass the 48 KB that need no opt-in.
 cudaError_t raise_smem_limit(const void* kernel, size_t smem, size_t optin);
 cudaError_t launch_reduce_partials(const KArgs& a, cudaStream_t st);
-cudaError_t set_forward_smem_limit(int op, int block, int items, int occ, size_t optin);
-cudaError_t set_backward_smem_limit(int block, int occ, int kind, size_t optin);
+cudaError_t set_forward_smem_limit(int op, int block, int items, int occ, size_t smem,
+                                   size_t optin);
+cudaError_t set_backward_smem_limit(int block, int occ, int kind, size_t smem, size_t optin);
 cudaError_t forward_occupancy(int op, int block, int items, int occ, size_t smem, int* ctas);
 cudaError_t backward_occupancy(int block, int occ, int kind, size_t smem, int* ctas);
 // direction vector-Jacobian products (a.grad_wi / a.grad_wo)
-cudaError_t set_dirgrad_smem_limit(int block, size_t optin);
+cudaError_t set_dirgrad_smem_limit(int block, size_t smem, size_t optin);
 cudaError_t dirgrad_occupancy(int block, size_t smem, int* ctas);
 cudaError_t launch_dirgrad(const KArgs& a, int block, int grid, size_t smem, cudaStream_t st);
 // test hook: the float path's own approximations beside CUDA's functions

@@ -44,3 +44,99 @@ for n in (680, 691, 692, 696, 699, 700, 702, 703, 704, 720):
 @pytest.mark.parametrize("shape", [(96, 80), (512, 256)])
 def test_traces_of_690_to_720_pieces(shape):
     _child(TRACE.format(shape=shape))
+
+# Tables of m bytes each (256 + 8 per texel), ascending.  Records in any order:
+# n_mat tables of m + 16 bytes and 20 warps' lists (12,800 bytes) for the
+# forward, n_mat times 8 to 15 sums and 16 warps' lists (18,432) for the
+# gradients; sorted records: a table slot per warp (20, or 16) and the lists.
+# All records are of material 0 and fit in one warp's round, so that every size
+# gives the same bits.
+CALLS = """
+n = 32
+rec = I.random_records(n, n_mat=1, seed=5, wi_mode="cosine", ratio={ratio}, sample=True)
+g = torch.from_numpy(np.random.default_rng(6).uniform(-1, 1, (3, n)).astype(np.float32)).cuda()
+
+def calls(M, d):
+    op = {op!r}
+    if op == "eval":
+        return api.eval(M, d)
+    if op == "sample":
+        return api.sample(M, d)
+    if op == "pdf":
+        return api.pdf(M, d)
+    if op == "fused":
+        return list(api.eval_sample_pdf(M, d).values())
+    if op == "stochastic":
+        return api.eval_stochastic(M, d, 3, 3)
+    if op == "backward":
+        return [api.eval_backward(M, d, g)[0]]
+    if op == "l2":
+        r = api.eval_l2_backward(M, d, g)
+        return [r[0][0], r[1][0], r[2]]
+    if op == "ext":
+        r = api.eval_backward_ext(M, d, g, dirs=True)
+        return [r[0][0], r[1], r[2]]
+
+want = None
+for n_mat, texels in {sizes}:
+    M = api.Materials([I.material(map_texels=texels)] * n_mat)
+    seg = np.array([0] + [n] * n_mat, np.int64) if {sort} else None
+    got = calls(M, api.records_to_device(rec, seg_offsets=seg))
+    torch.cuda.synchronize()
+    assert M.workspace_error() == 0
+    if {same_table}:
+        want = want or got
+        for a, b in zip(want, got):
+            assert torch.equal(a, b), (n_mat, texels)
+    else:
+        assert all(torch.isfinite(t).all() for t in got)
+"""
+
+
+@pytest.mark.parametrize("ratio", [None, "loguniform"])
+@pytest.mark.parametrize("op", ["eval", "sample", "pdf", "fused", "stochastic", "backward", "l2",
+                                "ext"])
+def test_tables_around_48_kb_in_any_order(op, ratio):
+    # forward, 128 texels: 28 tables are 49,088 bytes of dynamic shared memory;
+    # gradients, 256 texels: 13 tables are 48,992 to 49,392
+    sizes = [(k, 128) for k in range(20, 33)] + [(k, 256) for k in range(10, 16)]
+    sizes = [s for s in sizes if (s[1] == 256) == (op in ("backward", "l2", "ext"))]
+    _child(CALLS.format(op=op, ratio=repr(ratio), sizes=sizes, sort=False, same_table=True))
+
+
+@pytest.mark.parametrize("op", ["eval", "sample", "pdf", "fused", "stochastic", "backward", "l2",
+                                "ext"])
+def test_table_slots_around_48_kb_of_sorted_records(op):
+    # 20 slots and lists pass 48 KB at 194 texels, 16 at 270, 16 slots at 350
+    sizes = [(2, t) for t in range(180, 364, 2)]
+    _child(CALLS.format(op=op, ratio=None, sizes=sizes, sort=True, same_table=False))
+
+
+LARGEST = """
+n = 32
+rec = I.random_records(n, n_mat=1, seed=5, wi_mode="cosine", sample=True)
+g = torch.ones(3, n, device="cuda")
+seg = np.array([0, n, n], np.int64)
+d = api.records_to_device(rec, seg_offsets=seg)
+for call in (lambda M: api.eval(M, d), lambda M: api.eval_sample_pdf(M, d),
+             lambda M: api.eval_stochastic(M, d, 3, 3), lambda M: api.eval_backward(M, d, g),
+             lambda M: api.eval_backward_ext(M, d, g, dirs=True)):
+    refused = []
+    for texels in range(820, 886, 2):
+        M = api.Materials([I.material(map_texels=texels, migration_maps=2)] * 2)
+        try:
+            call(M)
+            refused.append(False)
+        except RuntimeError as e:
+            assert "material table too large for shared memory" in str(e), (texels, e)
+            refused.append(True)
+        torch.cuda.synchronize()
+    assert not refused[0] and refused[-1] and refused == sorted(refused)
+"""
+
+
+def test_the_largest_tables_are_refused_before_a_launch():
+    # tables of 544 + 16 bytes per texel: 16 slots (874 texels), or slots and
+    # lists (834), are the 227 KB of a CTA, but not beside the kernel's static
+    # shared memory
+    _child(LARGEST)
