@@ -430,18 +430,23 @@ size_t order_bytes(int items) {
   return sizeof(uint32_t) * (32 * (size_t)items + kOrderBuckets);
 }
 
-// The shape of a forward call: the caller's (or the tuned) one when set,
-// else the default for the kind of records.  Material-sorted records keep a
-// table slot per warp: tables too large for 20 slots (and the kernel's static
-// shared memory, under 1 KB) take the 16-warp shape.
-bysdf_launch_config fwd_cfg(const bysdf_materials* m, int op, const bysdf_hits* h,
-                            bool stochastic = false) {
-  if (m->cfg_set[op] || !h) return m->cfg[op];
-  if (h->ratio) return footprint_default_cfg();
+// The shape of a forward call: the caller's (or the tuned) one when set, which
+// is taken as it stands, else the default for the kind of records, whose tiles
+// follow the batch (by_batch).  Material-sorted records keep a table slot per
+// warp: tables too large for 20 slots (and the kernel's static shared memory,
+// under 1 KB) take the 16-warp shape.
+struct FwdShape {
+  bysdf_launch_config c;
+  bool by_batch;
+};
+FwdShape fwd_shape(const bysdf_materials* m, int op, const bysdf_hits* h,
+                   bool stochastic = false) {
+  if (m->cfg_set[op] || !h) return {m->cfg[op], !m->cfg_set[op]};
+  if (h->ratio) return {footprint_default_cfg(), true};
   const bysdf_launch_config c = near_default_cfg();
   const bool fits = (size_t)(c.block / 32) * ((size_t)m->stride + order_bytes(c.items)) + 1024 <=
                     m->smem_optin;
-  return !stochastic && (!h->seg_offsets || fits) ? c : m->cfg[op];
+  return {!stochastic && (!h->seg_offsets || fits) ? c : m->cfg[op], true};
 }
 
 int check_hits(const bysdf_materials* m, const bysdf_hits* h, bool need_wo, int64_t n) {
@@ -598,10 +603,10 @@ int op_bits(int op) {
 // sto: the stochastic estimators (flags != 0), eval and fused ops only
 int run_forward(const bysdf_materials* m, int op, const bysdf_hits* h, const float* u0,
                 const float* u1, int64_t n, const bysdf_outputs& o, void* ws, size_t ws_bytes,
-                cudaStream_t st, const bysdf_launch_config& cfg, size_t ws_need = 0,
+                cudaStream_t st, const FwdShape& chosen, size_t ws_need = 0,
                 const bysdf_stochastic* sto = nullptr) {
   int bits = op_bits(op);
-  bysdf_launch_config c = cfg;
+  bysdf_launch_config c = chosen.c;
   if (sto && sto->flags) {
     if (sto->flags & ~(uint32_t)(BYSDF_STOCH_JITTER_NODES | BYSDF_STOCH_ROUGH_ENTRY))
       return fail(BYSDF_E_ARG, "unknown stochastic flags");
@@ -673,7 +678,7 @@ int run_forward(const bysdf_materials* m, int op, const bysdf_hits* h, const flo
     // take 432 us, of 8 486 us, of 2 490 us; at 36 of 8 1407 us, of 4 1446 us)
     const int64_t rounds = (n + 31) / 32;
     int items = c.items, tile = c.items;
-    if (h->ratio && !m->cfg_set[op]) {
+    if (h->ratio && chosen.by_batch) {
       tile = rounds < 3 * warps ? 1 : rounds < 6 * warps ? 2 : rounds < 12 * warps ? 4 : items;
       items = tile;
       // the stochastic kernels keep the tile of one round or of c.items they
@@ -684,7 +689,7 @@ int run_forward(const bysdf_materials* m, int op, const bysdf_hits* h, const flo
       }
     } else if (a.n_tiles < warps) {
       items = tile = 1;
-    } else if (!m->cfg_set[op] && !h->ratio && !(bits & OPF_STOCH) && rounds < 16 * warps) {
+    } else if (chosen.by_batch && !h->ratio && !(bits & OPF_STOCH) && rounds < 16 * warps) {
       // sorted near-field records, a few tiles per warp: shorter ones end
       // together, more of them cost draws and table copies (fused: 5 rounds a
       // warp 65.3 us in tiles of 4, 56.5 of 2, 58.4 of 1; 13 rounds 135, 129,
@@ -1030,7 +1035,7 @@ int bysdf_eval(const bysdf_materials* m, const bysdf_hits* hits, int64_t n, floa
   o.status = status;
   if (!m) return fail(BYSDF_E_ARG, "materials is NULL");
   return run_forward(m, BYSDF_OP_EVAL, hits, nullptr, nullptr, n, o, workspace, workspace_bytes,
-                     reinterpret_cast<cudaStream_t>(stream), fwd_cfg(m, BYSDF_OP_EVAL, hits));
+                     reinterpret_cast<cudaStream_t>(stream), fwd_shape(m, BYSDF_OP_EVAL, hits));
 }
 
 int bysdf_eval_noalloc(const bysdf_materials* m, const bysdf_hits* hits, int64_t n,
@@ -1057,7 +1062,7 @@ int bysdf_eval_noalloc(const bysdf_materials* m, const bysdf_hits* hits, int64_t
   o.pdf = pdf;
   o.status = status;
   return run_forward(m, BYSDF_OP_EVAL, hits, nullptr, nullptr, n, o, scratch,
-                     BYSDF_NOALLOC_SCRATCH_BYTES, st, fwd_cfg(m, BYSDF_OP_EVAL, hits), need);
+                     BYSDF_NOALLOC_SCRATCH_BYTES, st, fwd_shape(m, BYSDF_OP_EVAL, hits), need);
 }
 
 // ------------------------------------------------------ host pipeline -----
@@ -1239,7 +1244,7 @@ int bysdf_eval_sample_pdf_host(bysdf_host_pipeline* p, const bysdf_hits* hits, c
     o.pdf_s = s.pdf_s;
     o.lobe_status = s.lstat;
     int rc = run_forward(p->m, BYSDF_OP_FUSED, &dh, s.u0, s.u1, mcount, o, s.ws, p->ws_bytes,
-                         p->s_run, fwd_cfg(p->m, BYSDF_OP_FUSED, &dh));
+                         p->s_run, fwd_shape(p->m, BYSDF_OP_FUSED, &dh));
     if (rc) return rc;
     BY_CU(cudaEventRecord(p->run_done[k], p->s_run));
     BY_CU(cudaStreamWaitEvent(p->s_out, p->run_done[k], 0));
@@ -1279,7 +1284,7 @@ int bysdf_sample(const bysdf_materials* m, const bysdf_hits* hits, const float* 
   o.lobe_status = lobe_status;
   if (!m) return fail(BYSDF_E_ARG, "materials is NULL");
   return run_forward(m, BYSDF_OP_SAMPLE, hits, u0, u1, n, o, workspace, workspace_bytes,
-                     reinterpret_cast<cudaStream_t>(stream), fwd_cfg(m, BYSDF_OP_SAMPLE, hits));
+                     reinterpret_cast<cudaStream_t>(stream), fwd_shape(m, BYSDF_OP_SAMPLE, hits));
 }
 
 int bysdf_pdf(const bysdf_materials* m, const bysdf_hits* hits, int64_t n, float* pdf,
@@ -1289,7 +1294,7 @@ int bysdf_pdf(const bysdf_materials* m, const bysdf_hits* hits, int64_t n, float
   o.status = status;
   if (!m) return fail(BYSDF_E_ARG, "materials is NULL");
   return run_forward(m, BYSDF_OP_PDF, hits, nullptr, nullptr, n, o, workspace, workspace_bytes,
-                     reinterpret_cast<cudaStream_t>(stream), fwd_cfg(m, BYSDF_OP_PDF, hits));
+                     reinterpret_cast<cudaStream_t>(stream), fwd_shape(m, BYSDF_OP_PDF, hits));
 }
 
 int bysdf_eval_sample_pdf(const bysdf_materials* m, const bysdf_hits* hits, const float* u0,
@@ -1307,7 +1312,7 @@ int bysdf_eval_sample_pdf(const bysdf_materials* m, const bysdf_hits* hits, cons
   o.lobe_status = lobe_status_s;
   if (!m) return fail(BYSDF_E_ARG, "materials is NULL");
   return run_forward(m, BYSDF_OP_FUSED, hits, u0, u1, n, o, workspace, workspace_bytes,
-                     reinterpret_cast<cudaStream_t>(stream), fwd_cfg(m, BYSDF_OP_FUSED, hits));
+                     reinterpret_cast<cudaStream_t>(stream), fwd_shape(m, BYSDF_OP_FUSED, hits));
 }
 
 int bysdf_trace_yarns(const bysdf_yarn* yarns, int32_t n_yarns, const bysdf_rays* rays,
@@ -1366,7 +1371,7 @@ int bysdf_eval_stochastic(const bysdf_materials* m, const bysdf_hits* hits,
   o.status = status;
   return run_forward(m, BYSDF_OP_EVAL, hits, nullptr, nullptr, n, o, workspace, workspace_bytes,
                      reinterpret_cast<cudaStream_t>(stream),
-                     fwd_cfg(m, BYSDF_OP_EVAL, hits, sto->flags != 0), 0, sto);
+                     fwd_shape(m, BYSDF_OP_EVAL, hits, sto->flags != 0), 0, sto);
 }
 
 int bysdf_eval_sample_pdf_stochastic(const bysdf_materials* m, const bysdf_hits* hits,
@@ -1387,7 +1392,7 @@ int bysdf_eval_sample_pdf_stochastic(const bysdf_materials* m, const bysdf_hits*
   o.lobe_status = lobe_status_s;
   return run_forward(m, BYSDF_OP_FUSED, hits, u0, u1, n, o, workspace, workspace_bytes,
                      reinterpret_cast<cudaStream_t>(stream),
-                     fwd_cfg(m, BYSDF_OP_FUSED, hits, sto->flags != 0), 0, sto);
+                     fwd_shape(m, BYSDF_OP_FUSED, hits, sto->flags != 0), 0, sto);
 }
 
 int bysdf_eval_backward(const bysdf_materials* m, const bysdf_hits* hits, int64_t n,
@@ -1555,7 +1560,8 @@ int bysdf_autotune(bysdf_materials* m, int op, const bysdf_hits* hits, const flo
     if (op == BYSDF_OP_BACKWARD)
       return run_backward(m, hits, n, grad_f, out->grad_params, 0, workspace, workspace_bytes,
                           st, c);
-    return run_forward(m, op, hits, u0, u1, n, *out, workspace, workspace_bytes, st, c);
+    return run_forward(m, op, hits, u0, u1, n, *out, workspace, workspace_bytes, st,
+                       FwdShape{c, false});
   };
   float best_ms = 1e30f;
   bysdf_launch_config best_c = m->cfg[op];

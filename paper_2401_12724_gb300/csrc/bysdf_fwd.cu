@@ -56,7 +56,9 @@ cudaError_t forward_occupancy(int op, int block, int items, int occ, size_t smem
 cudaError_t launch_forward(int op, const KArgs& a, int block, int items, int occ, int grid,
                            size_t smem, cudaStream_t st) {
   const void* f = fwd_fn(op, block, items, occ);
-  if (!f) return cudaErrorInvalidValue;
+  // a warp works on 32 * items records of its tile: a longer tile's others
+  // would be left out
+  if (!f || a.tile > 32 * items || a.tail > 32 * items) return cudaErrorInvalidValue;
   void* args[] = {const_cast<KArgs*>(&a)};
   return cudaLaunchKernel(f, dim3(grid), dim3(block), args, smem, st);
 }
