@@ -366,10 +366,12 @@ int bysdf_plain(int op, const bysdf_materials* m, const bysdf_hits* hits,
  * footprint (a shape of its own that cannot be set; 512 x 4 at occupancy 0
  * for the stochastic calls and for sorted records whose tables leave no room
  * for 20 warps) and 256 x 8 at occupancy 1 for records with a ratio plane (up
- * to 16 geometry nodes each); once set, the shape serves both kinds.  get
- * returns the set shape, else 512 x 4 (the backward: 512 x 8). */
+ * to 16 geometry nodes each); once set, the shape serves both kinds, until
+ * reset goes back to these defaults.  get returns the set shape, else 512 x 4
+ * (the backward: 512 x 8). */
 int bysdf_set_launch_config(bysdf_materials* m, int op, const bysdf_launch_config* cfg);
 int bysdf_get_launch_config(const bysdf_materials* m, int op, bysdf_launch_config* cfg);
+int bysdf_reset_launch_config(bysdf_materials* m, int op);
 
 /* Output buffers of one op, for bysdf_autotune (unused ones may be NULL). */
 typedef struct bysdf_outputs {
@@ -412,9 +414,11 @@ int bysdf_plain_fused(const bysdf_materials* m, const bysdf_hits* hits,
                       const int64_t* seg_offsets_host, const float* u0, const float* u1,
                       int64_t n, const bysdf_outputs* out, void* stream);
 
-/* Time every launch shape that can be set for op (BYSDF_OP_EVAL, _SAMPLE, _PDF,
- * _FUSED, _BACKWARD) on these records with CUDA events on `stream`, keep the
- * fastest in the table for later calls and return it in *best.  Writes the
+/* Time the defaults and every launch shape that can be set for op
+ * (BYSDF_OP_EVAL, _SAMPLE, _PDF, _FUSED, _BACKWARD) on these records with CUDA
+ * events on `stream` and keep the fastest in the table for later calls: a set
+ * shape, or the defaults, as after bysdf_reset_launch_config.  *best is what
+ * bysdf_get_launch_config returns from then on.  Writes the
  * op's outputs (several times).  Synchronises the stream; not capturable. */
 int bysdf_autotune(bysdf_materials* m, int op, const bysdf_hits* hits, const float* u0,
                    const float* u1, const float* grad_f, int64_t n, const bysdf_outputs* out,

@@ -92,6 +92,7 @@ SYMBOLS = [
      [P, C.POINTER(Hits), P, P, P, C.c_int64, C.POINTER(Outputs), P]),
     ("bysdf_set_launch_config", C.c_int, [P, C.c_int, C.POINTER(LaunchConfig)]),
     ("bysdf_get_launch_config", C.c_int, [P, C.c_int, C.POINTER(LaunchConfig)]),
+    ("bysdf_reset_launch_config", C.c_int, [P, C.c_int]),
     ("bysdf_autotune", C.c_int, [P, C.c_int, C.POINTER(Hits), P, P, P, C.c_int64,
                                  C.POINTER(Outputs), P, C.c_size_t, P, C.POINTER(LaunchConfig)]),
     ("bysdf_workspace_error", C.c_int, [P, P, C.POINTER(C.c_uint32)]),

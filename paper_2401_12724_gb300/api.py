@@ -128,6 +128,10 @@ class Materials:
         c = N.LaunchConfig(block, items, ctas_per_sm, occupancy)
         N.check(self.lib.bysdf_set_launch_config(self.handle, op, C.byref(c)), "set_launch_config")
 
+    def reset_launch_config(self, op: int):
+        """Back to the defaults, which follow the kind and number of records."""
+        N.check(self.lib.bysdf_reset_launch_config(self.handle, op), "reset_launch_config")
+
     def launch_config(self, op: int) -> dict:
         c = N.LaunchConfig()
         N.check(self.lib.bysdf_get_launch_config(self.handle, op, C.byref(c)), "get_launch_config")
@@ -441,6 +445,8 @@ def plain_fused(mats: Materials, rec: dict, seg_host, u0=None, u1=None, stream=N
 
 def autotune(mats: Materials, op: int, rec: dict, out: dict | None = None, grad_f=None,
              stream=None) -> dict:
+    """Keeps the fastest launch shape of op for these records in the table
+    (bysdf_autotune): a set one, or the defaults; returns launch_config(op)."""
     n = _n(rec)
     dev = rec["h"].device
     o = out if out is not None else alloc_fused(n, dev)
