@@ -49,7 +49,10 @@ constexpr size_t kAllSmemMax = 48 * 1024;
 
 thread_local std::string g_err;
 
+// An error of the CUDA runtime is returned once: the runtime would also hand it
+// to the next call of this thread that asks for its last error.
 int fail(int code, const std::string& msg) {
+  if (code == BYSDF_E_CUDA) cudaGetLastError();
   g_err = msg;
   return code;
 }
@@ -1003,6 +1006,7 @@ int bysdf_destroy_materials(bysdf_materials* m) {
   if (!m) return BYSDF_OK;
   cudaDeviceSynchronize();
   if (m->d_table) cudaFree(m->d_table);
+  cudaGetLastError();  // what failed here (in a capture, say) is not another call's error
   delete m;
   return BYSDF_OK;
 }
@@ -1176,6 +1180,7 @@ int bysdf_host_pipeline_destroy(bysdf_host_pipeline* p) {
   if (p->s_run) cudaStreamDestroy(p->s_run);
   if (p->s_out) cudaStreamDestroy(p->s_out);
   if (p->dev) cudaFree(p->dev);
+  cudaGetLastError();  // as in bysdf_destroy_materials
   delete p;
   return BYSDF_OK;
 }
