@@ -5,6 +5,7 @@ import ctypes as C
 import importlib.util
 import os
 import threading
+import warnings
 
 from . import build as _build
 
@@ -137,14 +138,25 @@ def load(build_if_missing: bool = True):
             f = getattr(L, name)
             f.restype = res
             f.argtypes = args
-        if os.path.exists(_build.BINDING_PATH):
-            spec = importlib.util.spec_from_file_location("_bysdf_torch", _build.BINDING_PATH)
-            m = importlib.util.module_from_spec(spec)
-            spec.loader.exec_module(m)
-            m.bind({name: C.cast(getattr(L, name), C.c_void_p).value for name, _, _ in SYMBOLS})
-            calls = m
+        calls = _load_calls(L)
         _lib = L
         return _lib
+
+
+def _load_calls(L):
+    """The native call path for library L, or None (calls then go through ctypes,
+    to the same results) where it was not built or cannot be loaded."""
+    if not os.path.exists(_build.BINDING_PATH):
+        return None
+    try:
+        spec = importlib.util.spec_from_file_location("_bysdf_torch", _build.BINDING_PATH)
+        m = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(m)
+        m.bind({name: C.cast(getattr(L, name), C.c_void_p).value for name, _, _ in SYMBOLS})
+        return m
+    except Exception as e:
+        warnings.warn(f"the native call path was not loaded, calls go through ctypes: {e}")
+        return None
 
 
 def check(rc: int, what: str):

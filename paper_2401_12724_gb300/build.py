@@ -6,6 +6,7 @@ import os
 import subprocess
 import sys
 import threading
+import warnings
 from concurrent.futures import ThreadPoolExecutor
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -61,9 +62,18 @@ def _stale(lib: str, deps=None) -> bool:
 
 
 def _build_binding(force: bool) -> None:
+    """Builds the native call path of api.py.  The library does not need it (its
+    calls then go through ctypes), so a failure is a warning."""
     if not force and not _stale(BINDING_PATH,
                                 [BINDING_SRC, os.path.join(INCLUDE, "bysdf.h")]):
         return
+    try:
+        _compile_binding()
+    except Exception as e:  # no compiler, no headers, no torch
+        warnings.warn(f"the native call path was not built, calls go through ctypes: {e}")
+
+
+def _compile_binding() -> None:
     import sysconfig
 
     import torch
