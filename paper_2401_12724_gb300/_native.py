@@ -149,6 +149,8 @@ def _load_calls(L):
     if not os.path.exists(_build.BINDING_PATH):
         return None
     try:
+        if not _build.binding_matches():
+            raise ImportError("it was built for another torch or Python")
         spec = importlib.util.spec_from_file_location("_bysdf_torch", _build.BINDING_PATH)
         m = importlib.util.module_from_spec(spec)
         spec.loader.exec_module(m)

@@ -64,13 +64,31 @@ def _stale(lib: str, deps=None) -> bool:
 def _build_binding(force: bool) -> None:
     """Builds the native call path of api.py.  The library does not need it (its
     calls then go through ctypes), so a failure is a warning."""
-    if not force and not _stale(BINDING_PATH,
-                                [BINDING_SRC, os.path.join(INCLUDE, "bysdf.h")]):
-        return
     try:
-        _compile_binding()
+        if force or _stale(BINDING_PATH, [BINDING_SRC, os.path.join(INCLUDE, "bysdf.h")]) \
+                or not binding_matches():
+            _compile_binding()
     except Exception as e:  # no compiler, no headers, no torch
         warnings.warn(f"the native call path was not built, calls go through ctypes: {e}")
+
+
+def _abi() -> str:
+    """What the binding's object layouts and symbols follow beside its source."""
+    import sysconfig
+
+    import torch
+
+    return " ".join((torch.__version__, str(sysconfig.get_config_var("SOABI")),
+                     f"cxx11={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"))
+
+
+def binding_matches() -> bool:
+    """The built binding is this Python's and this torch's (its stamp says so)."""
+    try:
+        with open(BINDING_PATH + ".abi") as f:
+            return f.read() == _abi()
+    except OSError:
+        return False
 
 
 def _compile_binding() -> None:
@@ -91,7 +109,13 @@ def _compile_binding() -> None:
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"g++ failed for bysdf_torch.cpp:\n{r.stderr}")
+    with open(tmp + ".abi", "w") as f:
+        f.write(_abi())
+    # the binary goes first: one without its stamp is built again, never loaded
+    if os.path.exists(BINDING_PATH + ".abi"):
+        os.remove(BINDING_PATH + ".abi")
     os.replace(tmp, BINDING_PATH)
+    os.replace(tmp + ".abi", BINDING_PATH + ".abi")
 
 
 def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False,

@@ -68,3 +68,41 @@ def test_the_binding_is_built_and_loaded_here():
                         "N.load(); assert N.calls is not None"],
                        cwd=B.ROOT, capture_output=True, text=True)
     assert r.returncode == 0, r.stderr
+
+
+def _fake_compiler(monkeypatch, made):
+    def run(cmd, **kw):
+        made.append(cmd)
+        with open(cmd[cmd.index("-o") + 1], "w"):
+            pass
+        return subprocess.CompletedProcess(cmd, 0, "", "")
+    monkeypatch.setattr(B.subprocess, "run", run)
+
+
+def test_another_torch_builds_the_binding_again(elsewhere, monkeypatch):
+    import torch
+
+    made = []
+    _fake_compiler(monkeypatch, made)
+    B.build()
+    n = len(made)
+    B.build()
+    assert len(made) == n  # up to date
+    monkeypatch.setattr(torch, "__version__", "9.9.9+other")
+    B.build()
+    assert len(made) == n + 1 and made[-1][-1] == "-lc10_cuda"
+    os.remove(B.BINDING_PATH + ".abi")
+    B.build()
+    assert len(made) == n + 2
+
+
+def test_a_binding_for_another_torch_is_not_loaded(monkeypatch):
+    import torch
+
+    N.load()
+    monkeypatch.setattr(torch, "__version__", "9.9.9+other")
+    monkeypatch.setattr(N, "_lib", None)
+    monkeypatch.setattr(N, "calls", None)
+    with pytest.warns(UserWarning, match="another torch"):
+        N.load(build_if_missing=False)
+    assert N.calls is None
