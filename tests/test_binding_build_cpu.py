@@ -53,6 +53,7 @@ def test_a_failed_library_build_is_an_error(elsewhere, monkeypatch):
 def test_the_library_loads_beside_a_binding_that_does_not(monkeypatch, tmp_path):
     bad = tmp_path / "_bysdf_torch.so"
     bad.write_bytes(b"not a library")
+    (tmp_path / "_bysdf_torch.so.abi").write_text(B._abi())
     N.load()
     monkeypatch.setattr(B, "BINDING_PATH", str(bad))
     monkeypatch.setattr(N, "_lib", None)
