@@ -38,10 +38,8 @@ struct alignas(16) MatDev {
 static_assert(sizeof(MatDev) == 256, "MatDev must be 256 bytes");
 
 // Fiber migration map k >= 1 (Sec. 3.5): a 32-byte header, then T texels.
-// Map 0 is the regular ring whose constants live in MatDev.  The header lies
-// behind any number of texels, so it is aligned like one: an odd count leaves
-// no more than 8 bytes.
-struct MigMap {
+// Map 0 is the regular ring whose constants live in MatDev.
+struct alignas(16) MigMap {
   float m_over_2pi;     // M_k / (2 pi)
   float kf_hi, kf_lo;   // fiber phase rate in map periods per length, split
   float dkf;            // d kf / d alpha_f
@@ -50,22 +48,29 @@ struct MigMap {
   float aux;            // map 1 only: low part of 1 / segment length
 };
 static_assert(sizeof(MigMap) == 32, "MigMap must be 32 bytes");
-static_assert(sizeof(MatDev) % alignof(MigMap) == 0 && sizeof(float2) % alignof(MigMap) == 0,
-              "a MigMap lies behind MatDev and any number of texels");
+
+// Bytes of a map's texels, an even number of them, where a MigMap follows: its
+// header is loaded 16 bytes at a time.  (Headers of 8-byte alignment behind an
+// odd count instead: 2^24 fused records 1474 -> 1486 us, 2^26 sorted ones 5773
+// -> 5813 us, from two loads for one.)
+__host__ __device__ inline int mig_texel_bytes(int T) {
+  return (int)sizeof(float2) * ((T + 1) & ~1);
+}
+static_assert(sizeof(MatDev) % alignof(MigMap) == 0 &&
+                  2 * sizeof(float2) % alignof(MigMap) == 0,
+              "a MigMap lies behind MatDev and an even number of texels");
 
 // Bytes of one material: header, map 0, K_m - 1 migration maps, and (when
 // migrating) the map index of each of 256 consecutive segments.
 constexpr int kMigPeriod = 256;
 __host__ __device__ inline size_t mat_bytes(int T, int K) {
-  return sizeof(MatDev) + sizeof(float2) * (size_t)T +
-         (size_t)(K - 1) * (sizeof(MigMap) + sizeof(float2) * (size_t)T) +
-         (K > 1 ? (size_t)kMigPeriod : 0);
+  if (K == 1) return sizeof(MatDev) + sizeof(float2) * (size_t)T;
+  return sizeof(MatDev) + (size_t)K * mig_texel_bytes(T) + (size_t)(K - 1) * sizeof(MigMap) +
+         (size_t)kMigPeriod;
 }
 __host__ __device__ inline const MigMap* mig_map(const MatDev& m, int k) {
-  const uint8_t* base = reinterpret_cast<const uint8_t*>(&m) + sizeof(MatDev) +
-                        sizeof(float2) * (size_t)m.T;
-  return reinterpret_cast<const MigMap*>(base + (size_t)(k - 1) *
-                                                    (sizeof(MigMap) + sizeof(float2) * (size_t)m.T));
+  const int off = k * mig_texel_bytes(m.T) + (k - 1) * (int)sizeof(MigMap);
+  return reinterpret_cast<const MigMap*>(reinterpret_cast<const uint8_t*>(&m + 1) + off);
 }
 __host__ __device__ inline MigMap* mig_map(MatDev& m, int k) {
   return const_cast<MigMap*>(mig_map(static_cast<const MatDev&>(m), k));

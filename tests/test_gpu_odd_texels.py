@@ -1,5 +1,5 @@
-"""Migrating materials whose maps have an odd number of texels: a migration
-map's header then starts 8 bytes off a 16-byte boundary, in the device table
+"""Migrating materials whose maps have an odd number of texels: the texels behind
+which a migration map's header lies are padded to 16 bytes, in the device table
 and in shared memory.  Every kernel that reads it gives the oracle's values."""
 import numpy as np
 import pytest
