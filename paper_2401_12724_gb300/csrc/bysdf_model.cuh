@@ -206,7 +206,7 @@ __device__ __forceinline__ void node_geometry(const MatDev& m, const float2* map
   const int n_re = m.nit < 1 ? m.nit : 1;
   int best = -1, n_upd = m.nit;
   float t_start = 0.f;
-  {
+  {  // (its names end here)
     // Float pass over all plies, to pick the closest ply and count N_i.  The
     // ply centre c = R_c (cos, sin)(psi_k + 2 pi kp kappa t) enters an update
     // only through b = (X0 - c).e and perp = (X0 - c) x e, which are linear
@@ -407,14 +407,12 @@ __device__ __forceinline__ void node_geometry(const MatDev& m, const float2* map
     const float b = qx * wx + qy * wy;
     const float perp = qx * wy - qy * wx;
     const float disc = (Rp - perp) * (Rp + perp);
-    {
-      // predicated (no branch): the chord from its near end max(-b - sq, 0)
-      // to its far end s2 = sq - b, where the ray meets the disc ahead
-      const float sq = sqrtf(fmaxf(disc, 0.f));
-      const float s2 = sq - b;
-      const float chord = s2 - fmaxf(-b - sq, 0.f);
-      occ += (disc > 0.f && s2 > 0.f) ? chord : 0.f;
-    }
+    // predicated (no branch): the chord from its near end max(-b - sq, 0)
+    // to its far end s2 = sq - b, where the ray meets the disc ahead
+    const float sq = sqrtf(fmaxf(disc, 0.f));
+    const float s2 = sq - b;
+    const float chord = s2 - fmaxf(-b - sq, 0.f);
+    occ += (disc > 0.f && s2 > 0.f) ? chord : 0.f;
   }
   const float occ_all = occ * m.inv_2Rp + of;
   out.g = xexp(-(mv.sigma_s * occ_all));
@@ -486,11 +484,11 @@ __device__ __forceinline__ void geometry_k(const MatDev& m, const float2* map,
     }
     X0x *= m.R;
     X0y *= m.R;
+    // a node of several: its last update takes the hardware sin/cos too
+    // (the aggregate averages the nodes' frames)
     NodeGeo nd;
-      // a node of several: its last update takes the hardware sin/cos too
-      // (the aggregate averages the nodes' frames)
-      node_geometry<PLIES>(m, map, mv, X0x, X0y, ex, ey, q.v, kappa, wx, wy, s0v, c0v,
-                                 phase_f_v, nd, false, !near);
+    node_geometry<PLIES>(m, map, mv, X0x, X0y, ex, ey, q.v, kappa, wx, wy, s0v, c0v, phase_f_v,
+                         nd, false, !near);
     if (!nd.hit) continue;
     nhit += 1;
     nis += nd.ni;
