@@ -55,8 +55,8 @@ OPS = {
 # workload, per record; the records stream through once, so traffic scales
 # with the record count).  It is reported only while the kernel sources are
 # the ones captured (SHA-256 of FUSED_SOURCES).
-TRAFFIC_CAPTURE = dict(sources_sha256="07f29fb7cc8d35a65bad24fce53f029eea1404be7ea8e7c308d8f21570f80e8a",
-                       bytes_per_record=82.51,
+TRAFFIC_CAPTURE = dict(sources_sha256="6d483962537a744b8543c0ec6b178d3a11cacc39ff79a340766b5e033cac4bee",
+                       bytes_per_record=84.11,
                        summary="profiles/k_forward_fused_eval-sample-pdf_8mat.md")
 FP32_LANES_PER_SM = 128   # FP32 FMA lanes per SM (2 flops each)
 XU_LANES_PER_SM = 16      # special-function (MUFU) lanes per SM
@@ -503,7 +503,8 @@ def main():
                                      "'workloads'",
                             step="fused eval(+pdf at wo) + one importance sample per record",
                             l2="inputs larger than L2 (~0.8 GB of records per step)",
-                            launch="640 x 4, the default for records without a footprint",
+                            launch="640 x 4, the default for records without a footprint "
+                                   "(the library's get names the defaults 512 x 4)",
                             parallelism=f"records sharded, {ws} rank(s)"),
                 # one fused kernel per step: the records come in any order, so no
                 # tile-plan kernel runs (the ncu launch list of this step shows one)
